@@ -22,8 +22,11 @@ namespace {
 struct VarClass {      // one persistent replica launch: the work items of one step variant
     int variant;
     int item_begin, item_count;
-    int grid, threads;
+    int threads;
+    int resident;      // CTAs of this kernel that the GPU holds
+    int grid, grid_y, block;   // this chunk's CTAs and their threads (chunk_shapes)
     size_t smem;       // dynamic shared memory per CTA
+    size_t conf_off;   // its warps' part of the Eq. 5 scratch (elements)
 };
 struct ParClass {      // one parent-kernel launch: the parent warps of one tile
     int L, threads, grid;
@@ -80,6 +83,8 @@ struct bd_ctx {
     double* d_dpart = nullptr;          // [part_ring][bpart_stride][3]
     double* d_dbead = nullptr;          // [max_windows][sum N][3]
     double* d_rgz = nullptr;            // [max_windows][n_chains]
+    void* d_conf_scratch = nullptr;     // window-end bonds of the resident warps
+    size_t conf_elems = 0;
     double* d_tsf = nullptr;
     double* d_tsf_acc = nullptr;
     double* d_lam = nullptr;
@@ -89,7 +94,7 @@ struct bd_ctx {
     unsigned long long* d_overext = nullptr;
     int32_t* d_dev_err = nullptr;       // error bits set by kernels whose bounded waits gave up
     int64_t* d_evt_scratch = nullptr;
-    int32_t* d_queue = nullptr;         // one work-item counter per variant launch
+    int32_t* d_queue = nullptr;         // per variant launch queue_len() work-item counters, one a part
     // the step chunk as a CUDA graph: queue reset, parent kernels, one
     // persistent replica kernel per variant (parallel branches), and three
     // event records (start, after the parents, after the replicas)
@@ -511,9 +516,10 @@ bd_status plan(bd_ctx* ctx)
     const int threads = ctx->f64 ? persist_threads_f64() : persist_threads_f32();
     for (size_t k = 0; k < items.size(); ++k) {
         if (ctx->var_classes.empty() || ctx->var_classes.back().variant != items[k].variant)
-            ctx->var_classes.push_back(VarClass{items[k].variant, (int)k, 0, 0, threads, 0});
+            ctx->var_classes.push_back(VarClass{items[k].variant, (int)k, 0, threads, 0, 0, 1, 0, 0, 0});
         ctx->var_classes.back().item_count++;
     }
+    ctx->conf_elems = 0;
     for (VarClass& vc : ctx->var_classes) {
         if (variant_hi(vc.variant)) {          // one CTA per replica
             cudaError_t e = ctx->f64 ? hi_prepare_f64() : hi_prepare_f32();
@@ -522,8 +528,13 @@ bd_status plan(bd_ctx* ctx)
                 return fail(ctx, BD_E_CUDA, "hydrodynamic-interaction kernels: %s", cudaGetErrorString(e));
             }
             vc.threads = ctx->f64 ? hi_threads_f64(vc.variant == kHIBase) : hi_threads_f32(vc.variant == kHIBase);
-            vc.grid = vc.item_count;
             vc.smem = ctx->f64 ? hi_smem_f64(vc.variant == kHIBase) : hi_smem_f32(vc.variant == kHIBase);
+            int per_sm = 1;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &per_sm, ctx->f64 ? hi_replica_func_f64(vc.variant == kHIBase) : hi_replica_func_f32(vc.variant == kHIBase),
+                vc.threads, vc.smem);
+            if (e != cudaSuccess) cudaGetLastError();
+            vc.resident = std::max(1, per_sm) * ctx->n_sm;
             continue;
         }
         vc.smem = ctx->f64 ? persist_smem_f64(vc.variant) : persist_smem_f32(vc.variant);
@@ -534,9 +545,10 @@ bd_status plan(bd_ctx* ctx)
             cudaGetLastError();
             return fail(ctx, BD_E_CUDA, "occupancy of variant %d: %s", vc.variant, cudaGetErrorString(e));
         }
-        const int warps = threads / 32;
-        const int need = (vc.item_count + warps - 1) / warps;
-        vc.grid = std::max(1, std::min(need, per_sm * ctx->n_sm));
+        vc.resident = per_sm * ctx->n_sm;
+        vc.conf_off = ctx->conf_elems;
+        if (ctx->conf)
+            ctx->conf_elems += (size_t)vc.resident * (threads / 32) * kConfSlots * 3 * variant_tile(vc.variant);
     }
     // parent launches: one per tile; warps pack parents of equal lane count
     std::stable_sort(par.begin(), par.end());
@@ -616,9 +628,79 @@ StepParams base_params(const bd_ctx* ctx)
     return p;
 }
 
+// How many runs the W windows of a launch split into, given the work items
+// that run at the same time and how many of them the GPU holds at once
+// (places). With six units a place and more, splitting gains nothing: the
+// last warps run faster while others idle (1024 chains x 16 items, 6.7 a
+// place, 10 windows: 19.92 ms whole, 19.85 ms in 5 parts), and a warp pays
+// about 2 us to set a unit up and mixes the code of the two noise halves
+// (uneven chains, 10.5 a place: 8.2 ms whole, 8.6 ms split). Below that the
+// idle part of the last round shows: 4096 items, 1.7 a place, 4 windows:
+// 2.56 ms whole, 2.32 ms split. Chains with hydrodynamic interaction (a CTA a
+// unit, latency-bound: the last CTAs run no faster) take 24.
+int replica_parts(int64_t items, int64_t places, int64_t W, int64_t per_place)
+{
+    return (int)std::max<int64_t>(1, std::min(W, (per_place * places + items - 1) / items));
+}
+
+// Work-item counters of one replica launch: a chunk touches at most
+// chunk_windows + 1 windows, so it has at most that many parts.
+int64_t queue_len(const bd_ctx* ctx) { return ctx->chunk_windows + 1; }
+
+// Splits every replica launch of steps [t0, t0 + n) and sizes its grid. A
+// launch with more units than the GPU holds warps takes every SM and goes
+// through its parts in order. Smaller ones (few chains, or one of many
+// variants) run side by side, each with its share of the SMs by work, every
+// part with CTAs of its own that hold as few warps as that share allows: a
+// warp alone on its SM sub-partition steps fastest (the float64 chain of 20
+// beads: 1.2 ms for ten windows side by side, 18.7 ms one after another).
+void chunk_shapes(bd_ctx* ctx, int64_t t0, int64_t n, std::vector<StepParams>& rp)
+{
+    const int64_t S = ctx->cfg.window_steps;
+    const int64_t W = std::max<int64_t>(1, (t0 + n + S - 1) / S - t0 / S);
+    double total_work = 0.0;
+    int64_t total_units = 0, total_items = 0;
+    for (const VarClass& vc : ctx->var_classes)
+        if (!variant_hi(vc.variant)) total_items += vc.item_count;
+    for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
+        VarClass& vc = ctx->var_classes[k];
+        const bool hi = variant_hi(vc.variant);
+        const int64_t warps = hi ? 1 : vc.threads / 32;
+        const int parts = replica_parts(hi ? vc.item_count : total_items, vc.resident * warps, W, hi ? 24 : 6);
+        rp[k].win_per_part = (int32_t)((W + parts - 1) / parts);
+        rp[k].n_parts = (int32_t)((W + rp[k].win_per_part - 1) / rp[k].win_per_part);
+        if (hi) {
+            vc.grid = rp[k].n_parts * vc.item_count;
+            vc.grid_y = 1;
+            vc.block = vc.threads;
+            continue;
+        }
+        total_units += (int64_t)rp[k].n_parts * vc.item_count;
+        total_work += (double)rp[k].n_parts * vc.item_count * ctx->var_cost[vc.variant];
+    }
+    for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
+        VarClass& vc = ctx->var_classes[k];
+        if (variant_hi(vc.variant)) continue;
+        const int64_t most = vc.threads / 32, parts = rp[k].n_parts, units = parts * vc.item_count;
+        const double share = (double)units * ctx->var_cost[vc.variant] / total_work;
+        const int64_t ctas = total_units <= vc.resident ? units : std::max<int64_t>(1, (int64_t)(share * vc.resident));
+        int64_t warps = std::max<int64_t>(1, (units + ctas - 1) / ctas);
+        while (warps <= most && (vc.item_count + warps - 1) / warps * parts > ctas) ++warps;
+        if (warps <= most) {              // one unit a warp, every part its own CTAs
+            vc.grid_y = (int)parts;
+            vc.grid = (int)((vc.item_count + warps - 1) / warps);
+            vc.block = (int)(32 * warps);
+        } else {
+            vc.grid_y = 1;
+            vc.grid = (int)std::min<int64_t>((units + most - 1) / most, vc.resident);
+            vc.block = vc.threads;
+        }
+    }
+}
+
 // Kernel-node parameters of the chunk graph for one chunk [t0, t0 + n).
 // `pp` / `rp` hold one StepParams per node (kernelParams point into them).
-void chunk_params(const bd_ctx* ctx, int64_t t0, int64_t n, std::vector<StepParams>& pp,
+void chunk_params(bd_ctx* ctx, int64_t t0, int64_t n, std::vector<StepParams>& pp,
                   std::vector<StepParams>& rp)
 {
     StepParams p = base_params(ctx);
@@ -634,8 +716,10 @@ void chunk_params(const bd_ctx* ctx, int64_t t0, int64_t n, std::vector<StepPara
         const VarClass& vc = ctx->var_classes[k];
         rp[k].items = ctx->d_items + vc.item_begin;
         rp[k].n_items = vc.item_count;
-        rp[k].queue = ctx->d_queue + k;
+        rp[k].queue = ctx->d_queue + k * queue_len(ctx);
+        if (ctx->conf) rp[k].conf_scratch = (char*)ctx->d_conf_scratch + vc.conf_off * ctx->tsize;
     }
+    chunk_shapes(ctx, t0, n, rp);
 }
 
 cudaKernelNodeParams parent_node(const bd_ctx* ctx, size_t k, StepParams* pk, void** args)
@@ -665,8 +749,8 @@ cudaKernelNodeParams replica_node(const bd_ctx* ctx, size_t k, StepParams* rk, v
     else
         kp.func = const_cast<void*>(ctx->f64 ? persist_func_f64(vc.variant, ctx->conf)
                                              : persist_func_f32(vc.variant, ctx->conf));
-    kp.gridDim = dim3(vc.grid);
-    kp.blockDim = dim3(vc.threads);
+    kp.gridDim = dim3(vc.grid, vc.grid_y);
+    kp.blockDim = dim3(vc.block);
     kp.sharedMemBytes = (unsigned)vc.smem;
     kp.kernelParams = args;
     return kp;
@@ -731,7 +815,7 @@ bd_status build_graph(bd_ctx* ctx)
     ms.dst = ctx->d_queue;
     ms.value = 0;
     ms.elementSize = sizeof(int32_t);
-    ms.width = ctx->var_classes.size();
+    ms.width = ctx->var_classes.size() * queue_len(ctx);
     ms.height = 1;
     ms.pitch = 0;
     cudaGraphNode_t mnode;
@@ -916,6 +1000,7 @@ bd_status autotune_probe(bd_ctx* ctx, int probe_steps, std::vector<double>& cost
         p.items = titems;
         p.n_items = (int32_t)items.size();
         p.queue = tqueue;
+        p.n_parts = p.win_per_part = 1;
         p.S = 1 << 30;                 // no window starts or ends inside the probe
         p.t0 = 1;
         p.n_steps = probe_steps;
@@ -957,6 +1042,7 @@ bd_status replan(bd_ctx* ctx)
     const size_t old_items = ctx->h_items.size();
     const int64_t old_part = ctx->part_stride;
     const int64_t old_bpart = ctx->bpart_stride;
+    const size_t old_conf = ctx->conf_elems;
     const size_t old_queue = ctx->var_classes.size();
     bd_status s = plan(ctx);
     if (s != BD_OK) return s;
@@ -970,15 +1056,18 @@ bd_status replan(bd_ctx* ctx)
     if ((s = dalloc(ctx, (void**)&ctx->d_part, sizeof(double) * (size_t)ctx->part_ring * (size_t)ctx->part_stride)) != BD_OK)
         return s;
     if (ctx->conf) {
+        dfree(ctx, ctx->d_conf_scratch, std::max<size_t>(ctx->tsize * old_conf, 16));
+        ctx->d_conf_scratch = nullptr;
+        if ((s = dalloc(ctx, &ctx->d_conf_scratch, ctx->tsize * ctx->conf_elems)) != BD_OK) return s;
         dfree(ctx, ctx->d_dpart, std::max<size_t>(sizeof(double) * 3 * (size_t)ctx->part_ring * (size_t)old_bpart, 16));
         ctx->d_dpart = nullptr;
         if ((s = dalloc(ctx, (void**)&ctx->d_dpart, sizeof(double) * 3 * (size_t)ctx->part_ring *
                                                         (size_t)ctx->bpart_stride)) != BD_OK)
             return s;
     }
-    dfree(ctx, ctx->d_queue, std::max<size_t>(sizeof(int32_t) * old_queue, 16));
+    dfree(ctx, ctx->d_queue, std::max<size_t>(sizeof(int32_t) * queue_len(ctx) * old_queue, 16));
     ctx->d_queue = nullptr;
-    if ((s = dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * ctx->var_classes.size())) != BD_OK) return s;
+    if ((s = dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * queue_len(ctx) * ctx->var_classes.size())) != BD_OK) return s;
     return build_graph(ctx);
 }
 
@@ -1210,6 +1299,7 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
             BD_TRY(dalloc(ctx, (void**)&ctx->d_dpart, sizeof(double) * 3 * (size_t)ctx->part_ring *
                                                           (size_t)ctx->bpart_stride));
             BD_TRY(dalloc(ctx, (void**)&ctx->d_dbead, sizeof(double) * 3 * (size_t)W * (size_t)ctx->n_beads));
+            BD_TRY(dalloc(ctx, &ctx->d_conf_scratch, ctx->tsize * ctx->conf_elems));
             BD_TRY(dalloc(ctx, (void**)&ctx->d_rgz, sizeof(double) * (size_t)W * (size_t)C));
         }
         BD_TRY(dalloc(ctx, (void**)&ctx->d_tsf, sizeof(double) * (size_t)W * (size_t)M));
@@ -1226,7 +1316,7 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
             goto failed;
         }
         BD_TRY(dalloc(ctx, (void**)&ctx->d_evt_scratch, sizeof(int64_t) * (size_t)(event_blocks(M) + 1)));
-        BD_TRY(dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * ctx->var_classes.size()));
+        BD_TRY(dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * queue_len(ctx) * ctx->var_classes.size()));
         BD_TRY(build_graph(ctx));
         if (cfg->checkpoint_steps > 0) BD_TRY(adj_plan(ctx));
         {

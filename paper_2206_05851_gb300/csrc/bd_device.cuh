@@ -54,6 +54,9 @@ struct ItemDev {
 // Threads of every parent-kernel CTA and of every adjoint-kernel CTA (the
 // kernels size their shared tables by them).
 constexpr int kParentThreads = 64;
+// Replica bonds of a warp per spring of its tile (conf_scratch): 32 lanes of
+// one replica, or of two.
+constexpr int kConfSlots = 64;
 constexpr int kAdjThreads = 128;
 
 // One warp of the parent kernel: `count` parents, chains
@@ -78,7 +81,7 @@ struct StepParams {
     const ChainDev* chains;
     const ItemDev* items;       // replica kernel: warp work items, longest first
     int32_t n_items;
-    int32_t* queue;             // next unclaimed work item (zeroed before each launch)
+    int32_t* queue;             // [n_parts] work items claimed (zeroed before each launch)
     const int32_t* parent_items;  // parent kernel: chain ids
     const ParentWarp* parent_warps;  // parent kernel: warps of this launch
     int32_t n_parent_warps;
@@ -103,6 +106,10 @@ struct StepParams {
     int64_t part_stride, M;
     int32_t win_ring, pad_ring;  // windows one chunk touches (started or ended) + 1
     int64_t t0, n_steps;
+    // replica kernels: the launch's windows split into n_parts runs of
+    // win_per_part windows (item_range); every (item, part) is a unit of work
+    int32_t n_parts, win_per_part;
+    void* conf_scratch;         // T [warps][kConfSlots L][3] window-end bonds of a warp's replicas (Eq. 5)
     double dt, s_min;
     int32_t S, flags, thr_mask, bell_mask;
     uint32_t key0, key1;
@@ -110,6 +117,30 @@ struct StepParams {
     // from the kernel-parameter bank instead of occupying registers.
     uint32_t rk0[10], rk1[10];
 };
+
+// Steps [t0, t1) of part `part` of a replica launch. Every window's replicas
+// start from that window's own snapshot, so the windows of a launch are
+// independent work: part 0 runs from the launch's first step (inside a window
+// if the launch starts there), the others from a window start, and only the
+// last part holds the replicas' state at the end of the launch.
+struct StepRange {
+    uint32_t t0, t1;     // steps stay below 2^32
+    int32_t s_in, w;     // place of t0 in its window, and that window
+    bool last;
+};
+__device__ __forceinline__ StepRange item_range(const StepParams& p, int part)
+{
+    StepRange r;
+    const int64_t wf = p.t0 / p.S + (int64_t)part * p.win_per_part;
+    const int64_t a = part == 0 ? p.t0 : wf * p.S;
+    const int64_t e = (wf + p.win_per_part) * p.S, end = p.t0 + p.n_steps;
+    r.t0 = (uint32_t)a;
+    r.t1 = (uint32_t)(e < end ? e : end);
+    r.w = (int32_t)wf;
+    r.s_in = (int32_t)(a - wf * p.S);
+    r.last = part + 1 == p.n_parts;
+    return r;
+}
 
 // Adjoint (bd_adjoint.cuh): per chain, for the adjoint only.
 struct AdjChain {

@@ -609,14 +609,16 @@ template <typename T, bool FAST, int NTM> struct HITileEngine {
     __device__ __forceinline__ void end(Shared&, int32_t*) {}
 };
 
-// Replicas: one CTA per work item (one replica), the items of this launch in
-// p.items. Spawn from the window-start snapshot, S steps, one force sample per
+// Replicas: one CTA per work item (one replica) and part (a run of the
+// launch's windows), the items of this launch in p.items. Spawn from the window-start snapshot, S steps, one force sample per
 // spring at the window end into the replica's partial row (its group).
 template <typename T, bool FAST, typename E>
 __device__ __forceinline__ void hi_replica_body(const StepParams& p, typename E::Shared& sm)
 {
-    if ((int)blockIdx.x >= p.n_items) return;
-    const ItemDev it = p.items[blockIdx.x];
+    const int part = (int)blockIdx.x / p.n_items;
+    if (part >= p.n_parts) return;
+    const ItemDev it = p.items[(int)blockIdx.x - part * p.n_items];
+    const StepRange rg = item_range(p, part);
     const ChainDev ch = p.chains[it.chain];
     const int N = ch.N, nb = N - 1;
     const bool harmonic = ch.spring == BD_SPRING_HARMONIC || ch.spring == BD_SPRING_VWF;
@@ -631,13 +633,12 @@ __device__ __forceinline__ void hi_replica_body(const StepParams& p, typename E:
     eng.begin(sm, N, p.flags);
     T* state = reinterpret_cast<T*>(p.state) + (ch.state_off + (int64_t)kglob * nb) * 3;
     const T* snap = reinterpret_cast<const T*>(p.snap);
-    hi_load_bonds(sm, state, N);
+    if (rg.s_in != 0) hi_load_bonds(sm, state, N);
     int floored = 0;
-    int s_in = (int)(p.t0 % p.S);
-    int64_t w = p.t0 / p.S;
-    const int64_t t_end = p.t0 + p.n_steps;
+    int s_in = rg.s_in;
+    int64_t w = rg.w;
 #pragma unroll 1
-    for (int64_t t = p.t0; t < t_end; ++t) {
+    for (int64_t t = rg.t0; t < (int64_t)rg.t1; ++t) {
         if (s_in == 0) hi_load_bonds(sm, snap + ((w % p.win_ring) * p.M + ch.spr_off) * 3, N);
         floored += eng.step(sm, ch, k, kl, p, N, key, (uint32_t)it.chain + p.chain_base, (uint32_t)t, harmonic, lj);
         if (eng.failed()) break;
@@ -657,7 +658,7 @@ __device__ __forceinline__ void hi_replica_body(const StepParams& p, typename E:
         }
     }
     eng.end(sm, p.dev_err);
-    hi_store_bonds(sm, state, N);
+    if (rg.last) hi_store_bonds(sm, state, N);
     if (floored) atomicAdd(p.overext + it.chain, (unsigned long long)floored);
 }
 

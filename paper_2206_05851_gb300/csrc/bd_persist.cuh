@@ -1,5 +1,9 @@
-// The persistent replica kernels: every warp claims work items (chain,
-// replica group) from its launch's queue, longest first, until none is left.
+// The persistent replica kernels: every warp claims work units (a work item
+// - chain, replica group - over a run of the launch's windows) from its
+// launch's queue until none is left. The replicas of every window start from
+// that window's snapshot, so a launch's windows need not follow one another:
+// the host splits them so far that a small batch fills the GPU and the last
+// units of a large one end together (bd_api.cu: replica_parts).
 // Warps are independent - a warp's replicas, their window-end reduction and
 // their state never involve another warp - so chains of any bead and replica
 // count share a launch and the load balances at warp granularity. There is
@@ -44,17 +48,31 @@ __global__ void __launch_bounds__(Persist<T>::threads, 1) replica_persist_kernel
     uint4* ptab = reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(bd_smem) + SM::wsm_bytes) +
                   warp * SM::tab_per_warp;
     const int lane = threadIdx.x & 31;
-    for (;;) {
-        int idx = 0;
-        if (lane == 0) idx = atomicAdd(p.queue, 1);
-        idx = __shfl_sync(0xffffffffu, idx, 0);
-        if (idx >= p.n_items) break;
-        if constexpr (V >= kLJBase)
-            run_one_item<T, V - kLJBase, FAST, SM::tab, CONF, true>(p.items[idx], p, wsm, ptab);
-        else if constexpr (V >= kPairBase)
-            run_pair_item<V - kPairBase, SM::tab, CONF>(p.items[idx], p, wsm, ptab);
-        else
-            run_one_item<T, V, FAST, SM::tab, CONF>(p.items[idx], p, wsm, ptab);
+    T* conf = CONF ? reinterpret_cast<T*>(p.conf_scratch) +
+                         (int64_t)((blockIdx.y * gridDim.x + blockIdx.x) * (Persist<T>::threads / 32) + warp) *
+                             (kConfSlots * SM::L * 3)
+                   : nullptr;
+    // Parts: gridDim.y = n_parts for a small launch (every part has its own
+    // CTAs), 1 for a large one (every CTA goes through the parts in order).
+    // The part, and so the steps of its units, is the same for the whole CTA
+    // and follows from launch constants. (The claim stays at the top of its
+    // loop: below the item it cost the 7-spring pair tile 600 bytes of spills
+    // a thread and 6% of its speed.)
+#pragma unroll 1
+    for (int part = (int)blockIdx.y; part < p.n_parts; part += (int)gridDim.y) {
+        const StepRange rg = item_range(p, part);
+        for (;;) {
+            int idx = 0;
+            if (lane == 0) idx = atomicAdd(p.queue + part, 1);
+            idx = __shfl_sync(0xffffffffu, idx, 0);
+            if (idx >= p.n_items) break;
+            if constexpr (V >= kLJBase)
+                run_one_item<T, V - kLJBase, FAST, SM::tab, CONF, true>(p.items[idx], rg, p, wsm, ptab, conf);
+            else if constexpr (V >= kPairBase)
+                run_pair_item<V - kPairBase, SM::tab, CONF>(p.items[idx], rg, p, wsm, ptab, conf);
+            else
+                run_one_item<T, V, FAST, SM::tab, CONF>(p.items[idx], rg, p, wsm, ptab, conf);
+        }
     }
 }
 

@@ -50,8 +50,9 @@ namespace bdra {
 constexpr int kWarpScratch = 512;   // >= slots per warp x springs = P (N-1) <= 32 L
 
 // Eq. 5 diagnostics of a work item's replicas (one per lane run) at the end
-// of window w; their bonds were just stored at state_slot (slot base of the
-// lane's replica).
+// of window w; their bonds were just stored at state_slot (base of the lane's
+// replica in the warp's scratch: the windows of a launch run side by side, so
+// the replica's place in the state is not free for it).
 template <typename T, int L>
 __device__ __noinline__ void conformation_item(const ItemDev& it, const ChainDev& ch,
                                                const StepParams& p, int w, const T* state_slot,
@@ -92,8 +93,8 @@ __device__ __forceinline__ void warp_window_sum(const T* wsm, int nb, int count,
 // the step loop carries no trace of them. H: the noise half of every replica
 // of the item (known when all are odd or all even), or -1.
 template <typename T, int L, bool FAST, bool TAB, bool CONF, bool LJ, int H>
-__device__ __forceinline__ void run_one_item_h(const ItemDev& it, const StepParams& p, T* wsm,
-                                               uint4* ptab)
+__device__ __forceinline__ void run_one_item_h(const ItemDev& it, const StepRange& rg, const StepParams& p,
+                                               T* wsm, uint4* ptab, T* conf)
 {
     const ChainDev ch = p.chains[it.chain];
     const int nb = ch.N - 1;
@@ -119,14 +120,17 @@ __device__ __forceinline__ void run_one_item_h(const ItemDev& it, const StepPara
     T* state = reinterpret_cast<T*>(p.state) + (ch.state_off + (int64_t)kglob * nb) * 3;
     const T* snap = reinterpret_cast<const T*>(p.snap);
     T qx[L], qy[L], qz[L];
-    load_bonds<T, L>(qx, qy, qz, state, lc);
+    // the replica's state where the launch starts inside a window, else the
+    // snapshot (read again by the loop: an unconditional load costs nothing, a
+    // branch around it 12 registers on the 4-spring tile); a part after the
+    // first never reads the state that the last one writes
+    load_bonds<T, L>(qx, qy, qz, rg.s_in != 0 ? state : snap + ((int64_t)(rg.w % p.win_ring) * p.M + ch.spr_off) * 3, lc);
 
     int floored = 0;
-    int s_in = (int)(p.t0 % p.S);
-    int w = (int)(p.t0 / p.S);                      // window index (< 2^31)
-    const uint32_t t_end = (uint32_t)(p.t0 + p.n_steps);   // steps stay below 2^32
+    int s_in = rg.s_in;
+    int w = rg.w;                                   // window index (< 2^31)
 #pragma unroll 1
-    for (uint32_t t = (uint32_t)p.t0; t < t_end; ++t) {
+    for (uint32_t t = rg.t0; t < rg.t1; ++t) {
         if (s_in == 0)   // spawn: copy the halted parent (Sec. II)
             load_bonds<T, L>(qx, qy, qz, snap + ((int64_t)(w % p.win_ring) * p.M + ch.spr_off) * 3, lc);
         if constexpr (LJ)
@@ -150,13 +154,14 @@ __device__ __forceinline__ void run_one_item_h(const ItemDev& it, const StepPara
             warp_window_sum<T>(wsm, nb, it.rep_count,
                                p.part_hist + (int64_t)(w % p.win_ring) * p.part_stride + ch.part_off + (int64_t)it.group * nb);
             if (CONF && (p.flags & BD_FLAG_CONFORMATION)) {
-                store_bonds<T, L>(qx, qy, qz, state, lc);
-                conformation_item<T, L>(it, ch, p, w, state, sw, P, G, lc.bead0, active, kglob);
+                T* mine = conf + (sw < P ? sw : 0) * nb * 3;
+                store_bonds<T, L>(qx, qy, qz, mine, lc);
+                conformation_item<T, L>(it, ch, p, w, mine, sw, P, G, lc.bead0, active, kglob);
             }
             ++w;
         }
     }
-    store_bonds<T, L>(qx, qy, qz, state, lc);
+    if (rg.last) store_bonds<T, L>(qx, qy, qz, state, lc);
     if (floored) atomicAdd(p.overext + it.chain, (unsigned long long)floored);
     if (TAB) __syncwarp();     // every lane is done with ptab before the next item refills it
 }
@@ -167,12 +172,12 @@ __device__ __forceinline__ void run_one_item_h(const ItemDev& it, const StepPara
 // identical-noise runs all draw the parent's, half 0): the half is fixed
 // for the whole warp and compiled in.
 template <typename T, int L, bool FAST, bool TAB = false, bool CONF = false, bool LJ = false>
-__device__ __forceinline__ void run_one_item(const ItemDev& it, const StepParams& p, T* wsm,
-                                             uint4* ptab = nullptr)
+__device__ __forceinline__ void run_one_item(const ItemDev& it, const StepRange& rg, const StepParams& p, T* wsm,
+                                             uint4* ptab, T* conf)
 {
     const bool h1 = (p.flags & BD_FLAG_IDENTICAL_NOISE) == 0 && noise_half((uint32_t)it.rep_begin + 1u) == 1u;
-    if (h1) run_one_item_h<T, L, FAST, TAB, CONF, LJ, 1>(it, p, wsm, ptab);
-    else run_one_item_h<T, L, FAST, TAB, CONF, LJ, 0>(it, p, wsm, ptab);
+    if (h1) run_one_item_h<T, L, FAST, TAB, CONF, LJ, 1>(it, rg, p, wsm, ptab, conf);
+    else run_one_item_h<T, L, FAST, TAB, CONF, LJ, 0>(it, rg, p, wsm, ptab, conf);
 }
 
 // ---------------------------------------------------------------------------

@@ -28,10 +28,12 @@ namespace bdra {
 #endif
 enum { PK_UNIF = 1, PK_BM = 2, PK_SPRING = 4, PK_LAP = 8, PK_UPD = 16 };
 // 1: the per-bead noise work stays where it is written in the step loop (an
-// empty asm fence on the bead index); 0: the compiler may move it (measured
-// 1% faster with one generator call per replica pair; same results).
+// empty asm fence on the bead index); 0: the compiler may move it. Same
+// results; 1024 chains x 64 replicas of 100 beads, 1000 steps: 19.95 ms with
+// the fence, 20.02 ms without (16384 chains of 50 beads, 200 steps: 15.84
+// and 15.99 ms).
 #ifndef BD_PAIR_NOISE_FENCE
-#define BD_PAIR_NOISE_FENCE 0
+#define BD_PAIR_NOISE_FENCE 1
 #endif
 
 template <int GROUP>
@@ -222,7 +224,7 @@ __device__ __forceinline__ void step_bonds2(float2 (&qx)[L], float2 (&qy)[L], fl
 }
 
 // Eq. 5 diagnostics of a work item with two replicas per lane at the end of
-// window w; their bonds were just stored at sa / sb.
+// window w; their bonds were just stored at sa / sb (in the warp's scratch).
 template <int L>
 __device__ __noinline__ void conformation_pair(const ItemDev& it, const ChainDev& ch,
                                                const StepParams& p, int w, const float* sa,
@@ -251,8 +253,8 @@ __device__ __noinline__ void conformation_pair(const ItemDev& it, const ChainDev
 // in the Eq. 5 window-end diagnostics. SHARED: the lane's two replicas are a
 // noise pair (one generator call per bead and step).
 template <int L, bool TAB, bool CONF, bool SHARED>
-__device__ __forceinline__ void run_pair_item_k(const ItemDev& it, const StepParams& p, float* wsm,
-                                                uint4* ptab)
+__device__ __forceinline__ void run_pair_item_k(const ItemDev& it, const StepRange& rg, const StepParams& p,
+                                                float* wsm, uint4* ptab, float* conf)
 {
     const ChainDev ch = p.chains[it.chain];
     const int nb = ch.N - 1;
@@ -276,26 +278,28 @@ __device__ __forceinline__ void run_pair_item_k(const ItemDev& it, const StepPar
         __syncwarp();
     }
 
-    float* state = reinterpret_cast<float*>(p.state) + ch.state_off * 3;
-    float* sa = state + (int64_t)ka * nb * 3;
-    float* sb = state + (int64_t)kb * nb * 3;
+    float* sa = reinterpret_cast<float*>(p.state) + (ch.state_off + (int64_t)ka * nb) * 3;
+    float* sb = sa + 3 * nb;
     const float* snap = reinterpret_cast<const float*>(p.snap);
+    // the replicas' state where the launch starts inside a window, else the
+    // snapshot (see run_one_item_h)
+    const float* la = rg.s_in != 0 ? sa : snap + ((int64_t)(rg.w % p.win_ring) * p.M + ch.spr_off) * 3;
+    const float* lb = rg.s_in != 0 ? sb : la;
     float2 qx[L], qy[L], qz[L];
 #pragma unroll
     for (int j = 0; j < L; ++j) {
         const int i = lc.bead0 + j;
         const bool v = i < nb;
-        qx[j] = make_float2(v && act_a ? sa[3 * i] : 0.0f, v && act_b ? sb[3 * i] : 0.0f);
-        qy[j] = make_float2(v && act_a ? sa[3 * i + 1] : 0.0f, v && act_b ? sb[3 * i + 1] : 0.0f);
-        qz[j] = make_float2(v && act_a ? sa[3 * i + 2] : 0.0f, v && act_b ? sb[3 * i + 2] : 0.0f);
+        qx[j] = make_float2(v && act_a ? la[3 * i] : 0.0f, v && act_b ? lb[3 * i] : 0.0f);
+        qy[j] = make_float2(v && act_a ? la[3 * i + 1] : 0.0f, v && act_b ? lb[3 * i + 1] : 0.0f);
+        qz[j] = make_float2(v && act_a ? la[3 * i + 2] : 0.0f, v && act_b ? lb[3 * i + 2] : 0.0f);
     }
 
     int floored = 0;
-    int s_in = (int)(p.t0 % p.S);
-    int w = (int)(p.t0 / p.S);                      // window index (< 2^31)
-    const uint32_t t_end = (uint32_t)(p.t0 + p.n_steps);   // steps stay below 2^32
+    int s_in = rg.s_in;
+    int w = rg.w;                                   // window index (< 2^31)
 #pragma unroll 1
-    for (uint32_t t = (uint32_t)p.t0; t < t_end; ++t) {
+    for (uint32_t t = rg.t0; t < rg.t1; ++t) {
         if (s_in == 0) {  // spawn both replicas from the halted parent (Sec. II)
             const float* src = snap + ((int64_t)(w % p.win_ring) * p.M + ch.spr_off) * 3;
 #pragma unroll
@@ -324,19 +328,22 @@ __device__ __forceinline__ void run_pair_item_k(const ItemDev& it, const StepPar
             warp_window_sum<float>(wsm, nb, it.rep_count,
                                    p.part_hist + (int64_t)(w % p.win_ring) * p.part_stride + ch.part_off + (int64_t)it.group * nb);
             if (CONF && (p.flags & BD_FLAG_CONFORMATION)) {
+                float* ca = conf + (sw < P ? ra : 0) * nb * 3;
+                float* cb = conf + (sw < P ? rb : 0) * nb * 3;
 #pragma unroll
                 for (int j = 0; j < L; ++j) {
                     const int i = lc.bead0 + j;
                     if (i < nb) {
-                        if (act_a) { sa[3 * i] = qx[j].x; sa[3 * i + 1] = qy[j].x; sa[3 * i + 2] = qz[j].x; }
-                        if (act_b) { sb[3 * i] = qx[j].y; sb[3 * i + 1] = qy[j].y; sb[3 * i + 2] = qz[j].y; }
+                        if (act_a) { ca[3 * i] = qx[j].x; ca[3 * i + 1] = qy[j].x; ca[3 * i + 2] = qz[j].x; }
+                        if (act_b) { cb[3 * i] = qx[j].y; cb[3 * i + 1] = qy[j].y; cb[3 * i + 2] = qz[j].y; }
                     }
                 }
-                conformation_pair<L>(it, ch, p, w, sa, sb, sw, P, G, lc.bead0, act_a, act_b, ka, kb);
+                conformation_pair<L>(it, ch, p, w, ca, cb, sw, P, G, lc.bead0, act_a, act_b, ka, kb);
             }
             ++w;
         }
     }
+    if (rg.last)
 #pragma unroll
     for (int j = 0; j < L; ++j) {
         const int i = lc.bead0 + j;
@@ -354,14 +361,14 @@ __device__ __forceinline__ void run_pair_item_k(const ItemDev& it, const StepPar
 // replicas at even offsets), unless every replica draws the parent's noise.
 // The condition is the same for every lane of the warp.
 template <int L, bool TAB, bool CONF = false>
-__device__ __forceinline__ void run_pair_item(const ItemDev& it, const StepParams& p, float* wsm,
-                                              uint4* ptab)
+__device__ __forceinline__ void run_pair_item(const ItemDev& it, const StepRange& rg, const StepParams& p,
+                                              float* wsm, uint4* ptab, float* conf)
 {
     const bool shared = (it.rep_begin & 1) == 0 && (p.flags & BD_FLAG_IDENTICAL_NOISE) == 0;
     if (shared)
-        run_pair_item_k<L, TAB, CONF, true>(it, p, wsm, ptab);
+        run_pair_item_k<L, TAB, CONF, true>(it, rg, p, wsm, ptab, conf);
     else
-        run_pair_item_k<L, TAB, CONF, false>(it, p, wsm, ptab);
+        run_pair_item_k<L, TAB, CONF, false>(it, rg, p, wsm, ptab, conf);
 }
 
 }  // namespace bdra

@@ -1,0 +1,72 @@
+"""The windows of a launch run side by side (their replicas start from their own snapshots). One bd_step over many windows
+equals the same steps taken a window (or less) at a time, bit for bit: the noise is keyed by the step, not by the launch."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2206_05851_gb300 import bdra, inputs as I  # noqa: E402
+
+
+def _fene(n, r, flow=I.FLOW_SHEAR):
+    return I.Chain(n_beads=n, n_replicas=r, spring=I.SPRING_FENE, flow=flow, b=40.0, rate=0.5, f_c=0.5 * 40 ** 0.5, k0=1e-3, dx=0.2)
+
+
+def _globule(n, r, hi):
+    ch = I.collapsed_chain(r, n_beads=n)
+    ch.hi_a = 1.0 if hi else 0.0
+    return ch
+
+
+# few units a launch (each window its own CTAs), one unit, uneven variants side by side, more units than warps, RPY (both kernels)
+BATCHES = {
+    "one": [_fene(20, 16)],
+    "dumbbell": [_fene(2, 1)],
+    "uneven": [_fene(n, r) for n, r in ((3, 5), (17, 8), (50, 33), (61, 2), (100, 7), (230, 3), (500, 2))],
+    "many": [_fene(50, 24) for _ in range(160)],
+    "collapsed": [_globule(n, r, False) for n, r in ((8, 3), (50, 7), (120, 2))],
+    "rpy": [_globule(n, r, True) for n, r in ((7, 2), (50, 3), (60, 2))],
+}
+
+
+def _run(chains, calls, S, windows, prec, flags):
+    wl = I.custom(chains, 4e-5 if chains[0].spring == I.SPRING_HARMONIC else 1e-3, S, S * windows)
+    ctx = bdra.Context(chains, wl.dt, S, 11, I.initial_positions(wl, seed=5), precision=prec, max_windows=windows,
+                       thr_mask=7, bell_mask=7, flags=flags, stream=torch.cuda.current_stream().cuda_stream)
+    for n in calls:
+        ctx.step(n)
+    W = sum(calls) // S
+    out = [ctx.replica_average(w) for w in range(W)] + [ctx.time_average(w) for w in range(W)]
+    out.append(ctx.positions(True))
+    if calls[0] % S == 0:      # a call that ends inside a window adds its part of the hazard to the total there: another order of sums
+        out += ctx.kinetics()
+    if flags & bdra.BD_FLAG_CONFORMATION:
+        out += [a for w in range(W) for a in ctx.conformation(w)]
+    assert ctx.info().windows_done == W
+    ctx.close()
+    return out
+
+
+@pytest.mark.parametrize("conf", [False, True])
+@pytest.mark.parametrize("prec", [bdra.BD_PREC_FP32, bdra.BD_PREC_FP64])
+@pytest.mark.parametrize("batch", sorted(BATCHES))
+def test_windows_side_by_side_equal_one_at_a_time(batch, prec, conf):
+    chains = BATCHES[batch]
+    if batch == "many" and prec == bdra.BD_PREC_FP64:
+        chains = chains[:24]
+    S, W = (7, 9) if batch != "many" else (5, 4)
+    flags = bdra.BD_FLAG_CONFORMATION if conf else 0
+    one = _run(chains, [S] * W + [3], S, W + 1, prec, flags)
+    for calls in ([S * W + 3], [2, S * W + 1]):                # from a window start; from inside a window
+        # RPY positions are rebuilt from the stored bonds at the start of every call, so only equal calls give equal bits there
+        if batch == "rpy" and calls != [S * W + 3]:
+            continue
+        got = _run(chains, calls, S, W + 1, prec, flags)
+        want = one if calls[0] % S == 0 else one[:2 * W + 1] + one[2 * W + 4:]
+        for a, b in zip(want, got, strict=True):
+            if batch == "rpy":
+                tol = 1e-3 if prec == bdra.BD_PREC_FP32 else 1e-10
+                assert np.abs(a - b).max() <= tol * max(1.0, np.abs(a).max())
+            else:
+                np.testing.assert_array_equal(a, b)
