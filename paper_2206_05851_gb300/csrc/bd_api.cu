@@ -94,6 +94,8 @@ struct bd_ctx {
     unsigned long long* d_overext = nullptr;
     int32_t* d_dev_err = nullptr;       // error bits set by kernels whose bounded waits gave up
     int64_t* d_evt_scratch = nullptr;
+    const void* noise_rad = nullptr;    // the device's float64 noise tables (float64 contexts; shared)
+    const void* noise_ang = nullptr;
     int32_t* d_queue = nullptr;         // per variant launch queue_len() work-item counters, one a part
     // the step chunk as a CUDA graph: queue reset, parent kernels, one
     // persistent replica kernel per variant (parallel branches), and three
@@ -612,6 +614,8 @@ StepParams base_params(const bd_ctx* ctx)
     p.first_bell = ctx->d_first_bell;
     p.exp1 = ctx->d_exp1;
     p.overext = ctx->d_overext;
+    p.rad_tab = (const double*)ctx->noise_rad;
+    p.ang_tab = (const double2*)ctx->noise_ang;
     p.dev_err = ctx->d_dev_err;
     p.part_stride = ctx->part_stride;
     p.M = ctx->M;
@@ -917,6 +921,49 @@ bd_status upload(bd_ctx* ctx, T** dst, const std::vector<T>& v)
     return BD_OK;
 }
 
+// The float64 noise tables of a device (24 MB of constants), shared by its
+// float64 contexts: filled by the first one before it is handed out, freed
+// with the last one. The maps are never destroyed, so that a context closed
+// at process exit still finds them.
+struct SharedTables { void* rad = nullptr; void* ang = nullptr; int users = 0; };
+std::mutex& tables_mutex() { static std::mutex* m = new std::mutex; return *m; }
+std::map<int, SharedTables>& tables_map() { static auto* t = new std::map<int, SharedTables>; return *t; }
+
+bd_status acquire_tables(bd_ctx* ctx)
+{
+    std::lock_guard<std::mutex> lock(tables_mutex());
+    SharedTables& t = tables_map()[ctx->device];
+    if (t.users == 0) {
+        cudaError_t e = cudaMalloc(&t.rad, noise_rad_bytes());
+        if (e == cudaSuccess) e = cudaMalloc(&t.ang, noise_ang_bytes());
+        if (e == cudaSuccess) e = run_noise_tables(t.rad, t.ang, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);   // other streams may read them from here on
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            if (t.rad) cudaFree(t.rad);
+            if (t.ang) cudaFree(t.ang);
+            t = SharedTables();
+            return fail(ctx, e == cudaErrorMemoryAllocation ? BD_E_OOM : BD_E_CUDA, "noise tables: %s", cudaGetErrorString(e));
+        }
+    }
+    ++t.users;
+    ctx->noise_rad = t.rad;
+    ctx->noise_ang = t.ang;
+    return BD_OK;
+}
+
+void release_tables(bd_ctx* ctx)     // after the context's stream has drained
+{
+    if (!ctx->noise_rad) return;
+    ctx->noise_rad = ctx->noise_ang = nullptr;
+    std::lock_guard<std::mutex> lock(tables_mutex());
+    SharedTables& t = tables_map()[ctx->device];
+    if (--t.users > 0) return;
+    cudaFree(t.rad);
+    cudaFree(t.ang);
+    t = SharedTables();
+}
+
 void release(bd_ctx* ctx)
 {
     if (!ctx) return;
@@ -932,6 +979,7 @@ void release(bd_ctx* ctx)
     if (ctx->adj_stream) { cudaStreamDestroy(ctx->adj_stream); ctx->adj_stream = nullptr; }
     for (void* p : ctx->allocs) cudaFree(p);
     ctx->allocs.clear();
+    release_tables(ctx);
     cudaGetLastError();
 }
 
@@ -1267,6 +1315,7 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
     }
     for (int v = 0; v < kVariantCodes; ++v) ctx->var_cost[v] = default_variant_cost(v);
     BD_TRY(plan(ctx));
+    if (ctx->f64) BD_TRY(acquire_tables(ctx));
     {
         const int64_t M = ctx->M, C = cfg->n_chains, W = cfg->max_windows;
         std::vector<int32_t> spring_chain(M);

@@ -94,6 +94,9 @@ struct StepParams {
     int64_t* first_thr;         // [3][M]
     int64_t* first_bell;        // [3][M]
     const double* exp1;         // [3][M] Exp(1) thresholds
+    // float64 runs: Box-Muller's two functions of the 21-bit fields (NoiseTab)
+    const double* rad_tab;
+    const double2* ang_tab;
     unsigned long long* overext;  // [n_chains]
     int32_t* dev_err;           // error bits of kernels whose bounded waits gave up (BD_DEV_ERR_*)
     // conformation diagnostics of Eq. 5 (with BD_FLAG_CONFORMATION)
@@ -598,12 +601,61 @@ template <bool FAST> struct Normals<double, FAST> {
     }
 };
 
+// The float64 normals from tables. A radius sqrt(-2 ln u) and an angle's
+// cosine and sine have only 2^21 arguments each (21-bit fields), and float64
+// arithmetic runs at 1/64 of the float32 rate here: the library's log, sqrt
+// and sincospi took about 210 of a bead-step's 250 float64 instructions. So
+// rad[m] holds every radius (16 MB) and ang[i] the cosine and sine of the
+// first quadrant's 2^19 angles (8 MB; the other quadrants are exact
+// reflections, the points m + 1/2 being symmetric), both computed by bm_pair's
+// own expressions, so the normals are the same bits. The tables stay in L2;
+// a bead-step gathers two entries of each.
+struct NoiseTab {
+    static constexpr int kRad = 1 << 21, kAng = 1 << 19;
+    static __device__ __forceinline__ double flip(double v, uint32_t neg)
+    {
+        return __hiloint2double(__double2hiint(v) ^ (int)(neg << 31), __double2loint(v));
+    }
+    // r cos (WANT 1 or 3) and r sin (WANT 2 or 3) of Box-Muller pair PR
+    template <int PR, int WANT>
+    static __device__ __forceinline__ void pair(uint4 x, const StepParams& p, double& c, double& s)
+    {
+        const double r = __ldg(p.rad_tab + Fields21::m(x, 2 * PR));
+        const uint32_t a = Fields21::m(x, 2 * PR + 1), q = a >> 19, i = a & (kAng - 1);
+        const double* t = reinterpret_cast<const double*>(p.ang_tab + i);
+        if (WANT == 3) {
+            const double2 v = __ldg(p.ang_tab + i);
+            c = r * flip((q & 1u) ? v.y : v.x, (q ^ (q >> 1)) & 1u);
+            s = r * flip((q & 1u) ? v.x : v.y, q >> 1);
+        } else if (WANT == 1) {
+            c = r * flip(__ldg(t + (q & 1u)), (q ^ (q >> 1)) & 1u);
+        } else {
+            s = r * flip(__ldg(t + ((q & 1u) ^ 1u)), q >> 1);
+        }
+    }
+    template <int H>
+    static __device__ __forceinline__ void draw_h(uint4 x, const StepParams& p, double& z0, double& z1, double& z2)
+    {
+        double unused;
+        if (H == 0) {
+            pair<0, 3>(x, p, z0, z1);
+            pair<1, 1>(x, p, z2, unused);
+        } else {
+            pair<1, 2>(x, p, unused, z0);
+            pair<2, 3>(x, p, z1, z2);
+        }
+    }
+};
+
 // Draw with the half fixed at compile time (H = 0, 1) or read at run time
 // (H = -1: h).
 template <typename T, bool FAST, int H>
-__device__ __forceinline__ void draw_half(uint4 x, uint32_t h, T& z0, T& z1, T& z2)
+__device__ __forceinline__ void draw_half(uint4 x, uint32_t h, const StepParams& p, T& z0, T& z1, T& z2)
 {
-    if (H == 0) Normals<T, FAST>::template draw_h<0>(x, z0, z1, z2);
+    if constexpr (sizeof(T) == 8) {
+        if (H == 0 || (H < 0 && h == 0)) NoiseTab::draw_h<0>(x, p, z0, z1, z2);
+        else NoiseTab::draw_h<1>(x, p, z0, z1, z2);
+    } else if (H == 0) Normals<T, FAST>::template draw_h<0>(x, z0, z1, z2);
     else if (H == 1) Normals<T, FAST>::template draw_h<1>(x, z0, z1, z2);
     else Normals<T, FAST>::draw(x, h, z0, z1, z2);
 }
@@ -615,7 +667,7 @@ template <typename T, bool FAST, int H = -1>
 __device__ __forceinline__ void bead_noise_split(uint4 bp, uint3 sp, const StepParams& p, uint32_t h,
                                                  T& z0, T& z1, T& z2)
 {
-    draw_half<T, FAST, H>(PhiloxSplit::finish(bp, sp, p.rk0, p.rk1), h, z0, z1, z2);
+    draw_half<T, FAST, H>(PhiloxSplit::finish(bp, sp, p.rk0, p.rk1), h, p, z0, z1, z2);
 }
 
 // The normals of (bead, slot, step, chain) from the full generator.
@@ -625,7 +677,7 @@ __device__ __forceinline__ void bead_noise(uint32_t bead, uint32_t slot, uint32_
                                            T& z0, T& z1, T& z2)
 {
     const uint4 x = philox4x32_10_rk(make_uint4(bead, noise_word(slot), step, chain), p.rk0, p.rk1);
-    draw_half<T, FAST, H>(x, noise_half(slot), z0, z1, z2);
+    draw_half<T, FAST, H>(x, noise_half(slot), p, z0, z1, z2);
 }
 
 // ---------------------------------------------------------------------------

@@ -57,6 +57,11 @@ int hi_threads_f64(bool small);
 cudaError_t hi_prepare_f32();
 cudaError_t hi_prepare_f64();
 
+// The float64 noise tables (NoiseTab): sizes and the kernel that fills them.
+size_t noise_rad_bytes();
+size_t noise_ang_bytes();
+cudaError_t run_noise_tables(void* rad, void* ang, cudaStream_t st);
+
 // Parent kernels per tile; lj: the collapsed-chain step.
 const void* parent_func_f32(int L, bool lj);
 const void* parent_func_f64(int L, bool lj);

@@ -41,6 +41,30 @@ const void* persist_func_f64(int v, bool conf)
     return conf ? persist_conf_f64(v) : persist_plain_f64(v);
 }
 
+namespace {
+// NoiseTab's entries, by the expressions of bm_pair.
+__global__ void noise_tables_kernel(double* rad, double2* ang)
+{
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    const double u = ((double)m + 0.5) * 4.76837158203125e-7;      // (m + 1/2) 2^-21
+    if (m < NoiseTab::kRad) rad[m] = sqrt(-2.0 * log(u));
+    if (m < NoiseTab::kAng) {
+        double s, c;
+        sincospi(2.0 * u, &s, &c);
+        ang[m] = make_double2(c, s);
+    }
+}
+}  // namespace
+
+size_t noise_rad_bytes() { return sizeof(double) * NoiseTab::kRad; }
+size_t noise_ang_bytes() { return sizeof(double2) * NoiseTab::kAng; }
+
+cudaError_t run_noise_tables(void* rad, void* ang, cudaStream_t st)
+{
+    noise_tables_kernel<<<NoiseTab::kRad / 256, 256, 0, st>>>((double*)rad, (double2*)ang);
+    return cudaGetLastError();
+}
+
 int persist_threads_f64() { return Persist<double>::threads; }
 
 size_t persist_smem_f64(int v)

@@ -70,3 +70,26 @@ def test_windows_side_by_side_equal_one_at_a_time(batch, prec, conf):
                 assert np.abs(a - b).max() <= tol * max(1.0, np.abs(a).max())
             else:
                 np.testing.assert_array_equal(a, b)
+
+
+def test_float64_noise_tables_outlive_the_context_that_filled_them():
+    """The float64 contexts of a device share their noise tables: one closed early leaves the others' results unchanged, and
+    one opened after all were closed fills them again."""
+    chains = BATCHES["uneven"][:4]
+    want = _run(chains, [20], 10, 2, bdra.BD_PREC_FP64, 0)
+    wl = I.custom(chains, 1e-3, 10, 20)
+
+    def make():
+        return bdra.Context(chains, wl.dt, 10, 11, I.initial_positions(wl, seed=5), precision=bdra.BD_PREC_FP64, max_windows=2,
+                            stream=torch.cuda.current_stream().cuda_stream)
+
+    a, b = make(), make()
+    a.step(5)
+    a.close()
+    b.step(20)
+    np.testing.assert_array_equal(b.replica_average(1), want[1])
+    b.close()
+    c = make()
+    c.step(20)
+    np.testing.assert_array_equal(c.positions(True), want[4])
+    c.close()
