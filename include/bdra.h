@@ -262,8 +262,14 @@ bd_status bd_get_positions(bd_ctx* ctx, int32_t all_slots, double* out, int64_t*
  * history and kinetic state cleared. */
 bd_status bd_set_positions(bd_ctx* ctx, const double* pos, int64_t step);
 
-/* Counters and sizes (host struct). */
+/* Counters and sizes (host struct). Synchronises the stream. */
 bd_status bd_get_info(bd_ctx* ctx, bd_info* out);
+
+/* M, the length of a profile row (host int64), for callers that size their
+ * arrays before every read: unlike bd_get_info it does not wait for the
+ * stream, except in a context whose chains run the tensor-core kernels, where
+ * it reports BD_E_TIMEOUT as bd_get_info does. */
+bd_status bd_spring_count(bd_ctx* ctx, int64_t* n_springs);
 
 /* Autotuner of the launch shapes (the batching form of the method: chains of
  * uneven bead and replica counts share one persistent launch). For every

@@ -99,6 +99,7 @@ def load() -> ctypes.CDLL:
         "bd_get_positions": ([vp, ctypes.c_int32, vp, P(ctypes.c_int64)], st),
         "bd_set_positions": ([vp, vp, ctypes.c_int64], st),
         "bd_get_info": ([vp, P(bd_info)], st),
+        "bd_spring_count": ([vp, P(ctypes.c_int64)], st),
         "bd_autotune": ([vp, ctypes.c_int32, ctypes.c_int32], st),
         "bd_get_plan": ([vp, vp, vp, vp], st),
         "bd_enable_timing": ([vp, ctypes.c_int32], st),
@@ -207,13 +208,20 @@ def bd_get_info(ctx: int) -> bd_info:
     return info
 
 
+def bd_spring_count(ctx: int) -> int:
+    """M, without waiting for the stream (BD_E_TIMEOUT as bd_get_info for the tensor-core chains)."""
+    n = ctypes.c_int64(0)
+    _check(load().bd_spring_count(ctx, ctypes.byref(n)), ctx)
+    return int(n.value)
+
+
 def bd_replica_average(ctx: int, window: int, out) -> None:
-    M = bd_get_info(ctx).n_springs
+    M = bd_spring_count(ctx)
     _check(load().bd_replica_average(ctx, int(window), _need(out, 8 * M, "out")), ctx)
 
 
 def bd_time_average(ctx: int, window: int, out) -> None:
-    M = bd_get_info(ctx).n_springs
+    M = bd_spring_count(ctx)
     _check(load().bd_time_average(ctx, int(window), _need(out, 8 * M, "out")), ctx)
 
 
@@ -234,7 +242,7 @@ def bd_detect_events(ctx: int, out, capacity: int, log_surv=None) -> int:
 
 
 def bd_get_kinetics(ctx: int, hazard=None, first_thr=None, first_bell=None) -> None:
-    M = bd_get_info(ctx).n_springs
+    M = bd_spring_count(ctx)
     args = [_need(a, 24 * M, name) if a is not None else None
             for a, name in ((hazard, "hazard"), (first_thr, "first_thr"),
                             (first_bell, "first_bell"))]

@@ -1253,15 +1253,19 @@ bd_status adj_parents(bd_ctx* ctx, int kind, AdjParams a, cudaStream_t st)
 // Kernels whose bounded waits gave up leave bits in the context's device
 // error word (StepParams::dev_err); the calls below that synchronise the
 // stream report them as BD_E_TIMEOUT.
+bd_status device_error_status(bd_ctx* ctx, int32_t e)
+{
+    if (e)
+        return fail(ctx, BD_E_TIMEOUT, "a tensor-core completion wait gave up (device error bits 0x%x); "
+                    "the steps run since are not valid", (unsigned)e);
+    return BD_OK;
+}
 bd_status check_device_error(bd_ctx* ctx)
 {
     int32_t e = 0;
     BD_CUDA(ctx, cudaMemcpyAsync(&e, ctx->d_dev_err, sizeof(e), cudaMemcpyDeviceToHost, ctx->stream));
     BD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (e)
-        return fail(ctx, BD_E_TIMEOUT, "a tensor-core completion wait gave up (device error bits 0x%x); "
-                    "the steps run since are not valid", (unsigned)e);
-    return BD_OK;
+    return device_error_status(ctx, e);
 }
 
 }  // namespace
@@ -1364,7 +1368,7 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
             s = fail(ctx, BD_E_CUDA, "device error word");
             goto failed;
         }
-        BD_TRY(dalloc(ctx, (void**)&ctx->d_evt_scratch, sizeof(int64_t) * (size_t)(event_blocks(M) + 1)));
+        BD_TRY(dalloc(ctx, (void**)&ctx->d_evt_scratch, sizeof(int64_t) * (size_t)(event_blocks(M) + 2)));
         BD_TRY(dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * queue_len(ctx) * ctx->var_classes.size()));
         BD_TRY(build_graph(ctx));
         if (cfg->checkpoint_steps > 0) BD_TRY(adj_plan(ctx));
@@ -1517,31 +1521,32 @@ bd_status bd_detect_events(bd_ctx* ctx, bd_event* out, int64_t capacity, int64_t
     }
     ctx->launches += 3;
     BD_CUDA(ctx, run_events(ctx->d_chains, ctx->d_spring_chain, ctx->M, ctx->d_first_thr,
-                            ctx->d_first_bell, ctx->d_evt_scratch, dst, capacity, ctx->stream));
-    int64_t total = 0;
-    BD_CUDA(ctx, cudaMemcpyAsync(&total, ctx->d_evt_scratch + nblk, sizeof(int64_t),
-                                 cudaMemcpyDeviceToHost, ctx->stream));
+                            ctx->d_first_bell, ctx->d_evt_scratch, ctx->d_dev_err, dst, capacity, ctx->stream));
+    const bool ldev = log_surv && is_device_ptr(log_surv);
+    if (ldev) {          // before the one wait of this call
+        ++ctx->launches;
+        BD_CUDA(ctx, run_log_survival(ctx->d_chains, ctx->cfg.n_chains, ctx->M, ctx->d_lam, log_surv, ctx->stream));
+    }
+    int64_t seen[2] = {0, 0};        // events, device error bits
+    BD_CUDA(ctx, cudaMemcpyAsync(seen, ctx->d_evt_scratch + nblk, sizeof(seen), cudaMemcpyDeviceToHost, ctx->stream));
     BD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    const int64_t total = seen[0];
     if (capacity > 0 && !dev)
         BD_CUDA(ctx, cudaMemcpy(out, dst, sizeof(bd_event) * (size_t)std::min(total, capacity),
                                 cudaMemcpyDeviceToHost));
-    if (log_surv) {
-        const bool ldev = is_device_ptr(log_surv);
-        double* ld = log_surv;
+    if (log_surv && !ldev) {
         const size_t n = sizeof(double) * 3 * (size_t)ctx->cfg.n_chains;
-        if (!ldev) {
-            s = ensure_io(ctx, n);
-            if (s != BD_OK) return s;
-            ld = (double*)ctx->d_io;
-        }
+        s = ensure_io(ctx, n);
+        if (s != BD_OK) return s;
+        double* ld = (double*)ctx->d_io;
         ++ctx->launches;
         BD_CUDA(ctx, run_log_survival(ctx->d_chains, ctx->cfg.n_chains, ctx->M, ctx->d_lam, ld,
                                       ctx->stream));
-        s = deliver(ctx, log_surv, ld, n, ldev);
+        s = deliver(ctx, log_surv, ld, n, false);
         if (s != BD_OK) return s;
     }
     *n_out = total;
-    s = check_device_error(ctx);
+    s = device_error_status(ctx, (int32_t)seen[1]);
     if (s != BD_OK) return s;
     if (total > capacity)
         return fail(ctx, BD_E_CAPACITY, "%lld events, capacity %lld", (long long)total,
@@ -1625,6 +1630,20 @@ bd_status bd_get_info(bd_ctx* ctx, bd_info* out)
     out->kernel_launches = ctx->launches;
     out->n_launch_classes = (int32_t)(ctx->var_classes.size() + ctx->par_classes.size());
     out->precision = ctx->cfg.precision;
+    return BD_OK;
+}
+
+bd_status bd_spring_count(bd_ctx* ctx, int64_t* n_springs)
+{
+    if (!ctx) return BD_E_INVALID;
+    if (!n_springs) return fail(ctx, BD_E_INVALID, "n_springs is NULL");
+    for (const VarClass& vc : ctx->var_classes)
+        if (vc.variant == kHIBase && !ctx->f64) {          // the tensor-core kernels: the only ones that wait
+            const bd_status s = check_device_error(ctx);
+            if (s != BD_OK) return s;
+            break;
+        }
+    *n_springs = ctx->M;
     return BD_OK;
 }
 

@@ -26,7 +26,7 @@ cudaError_t run_window_criteria(const ChainDev* chains, const int32_t* spring_ch
 int64_t event_blocks(int64_t M);
 cudaError_t run_events(const ChainDev* chains, const int32_t* spring_chain, int64_t M,
                        const int64_t* first_thr, const int64_t* first_bell, int64_t* block_scratch,
-                       bd_event* out, int64_t capacity, cudaStream_t st);
+                       const int32_t* dev_err, bd_event* out, int64_t capacity, cudaStream_t st);
 cudaError_t run_log_survival(const ChainDev* chains, int n_chains, int64_t M, const double* lam,
                              double* out, cudaStream_t st);
 cudaError_t run_adj_seed(const ChainDev* chains, const int32_t* spring_chain, int64_t M,
