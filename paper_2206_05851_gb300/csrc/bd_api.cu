@@ -33,6 +33,7 @@ struct ParClass {      // one parent-kernel launch: the parent warps of one tile
     int warp_begin, warp_count;
     bool lj;           // collapsed chains (harmonic springs, pair forces)
     bool hi;           // hydrodynamic interaction: one CTA per parent
+    bool block;        // few parents: parent_block_kernel, one CTA per warp of parents
     size_t smem;
 };
 constexpr int kParentLJKey = 1000;   // planner key offset of the collapsed-chain parents
@@ -353,6 +354,26 @@ int choose_parent_tile(int N)
     return 0;
 }
 
+// Warps of free-draining Hooke and FENE parents, with tiles of at least
+// `least` springs a lane (parents of equal lane count share a warp).
+int64_t parent_warps_at(const bd_ctx* ctx, int least)
+{
+    std::map<std::pair<int, int>, int64_t> of;
+    for (const bd_chain_desc& d : ctx->chains) {
+        if (d.hi_a > 0 || d.spring == BD_SPRING_HARMONIC || d.spring == BD_SPRING_VWF) continue;
+        const int L = least <= 1 && d.n_beads <= 32 ? 1 : choose_parent_tile(d.n_beads);
+        ++of[{L, (d.n_beads + L - 1) / L}];
+    }
+    int64_t warps = 0;
+    for (const auto& x : of) warps += (x.second + 32 / x.first.second - 1) / (32 / x.first.second);
+    return warps;
+}
+// Up to how many warps of parents an SM the block kernel is the faster one
+// (us a step): 64 float64 chains of 100 beads 27.5 -> 4.8, 256 float32 chains
+// of 100 beads 1.11 -> 0.65, 512 of 20 to 500 beads 7.1 -> 2.8; 1024 of 100
+// beads 1.34 -> 1.45, 16384 of 50 beads with every criterion 7.2 -> 14.8.
+constexpr int kParentBlockWarps = 5;
+
 bd_status validate(bd_ctx* ctx, const bd_config* cfg)
 {
     if (!cfg) return fail(ctx, BD_E_INVALID, "cfg is NULL");
@@ -553,6 +574,15 @@ bd_status plan(bd_ctx* ctx)
             ctx->conf_elems += (size_t)vc.resident * (threads / 32) * kConfSlots * 3 * variant_tile(vc.variant);
     }
     // parent launches: one per tile; warps pack parents of equal lane count
+    // (parents of Hooke and FENE chains: of at most kParentBlockWarps warps an
+    // SM, the block kernel, in float64 with one bead a lane where that keeps them
+    // so few: a float64 instruction takes the pipe as long for 10 lanes as for
+    // 20, one chain of 20 beads steps in 1.3 us instead of 2.3)
+    const bool few = parent_warps_at(ctx, 2) <= kParentBlockWarps * (int64_t)ctx->n_sm;
+    if (few && ctx->f64 && cfg.checkpoint_steps == 0 && parent_warps_at(ctx, 1) <= kParentBlockWarps * (int64_t)ctx->n_sm)
+        for (auto& k : par)
+            if (k.first.first < kParentLJKey && ctx->chains[k.second].n_beads <= 32)
+                k.first = {1, ctx->chains[k.second].n_beads};
     std::stable_sort(par.begin(), par.end());
     ctx->h_parent_items.clear();
     ctx->h_parent_warps.clear();
@@ -563,11 +593,12 @@ bd_status plan(bd_ctx* ctx)
         const int P = hi ? 1 : 32 / G;           // one CTA per parent with hydrodynamic interaction
         const int L = hi ? key - kParentHIKey : key % kParentLJKey;   // hi: 0 small, 1 large chains
         const bool lj = !hi && key >= kParentLJKey;
+        const bool block = few && !hi && !lj;
         if (ctx->par_classes.empty() || ctx->par_classes.back().L != L || ctx->par_classes.back().lj != lj ||
             ctx->par_classes.back().hi != hi)
             ctx->par_classes.push_back(ParClass{L, hi ? (ctx->f64 ? hi_threads_f64(L == 0) : hi_threads_f32(L == 0))
-                                                      : kParentThreads, 0,
-                                                (int)ctx->h_parent_warps.size(), 0, lj, hi,
+                                                      : block ? kParentThreads2 : kParentThreads, 0,
+                                                (int)ctx->h_parent_warps.size(), 0, lj, hi, block,
                                                 hi ? (ctx->f64 ? hi_smem_f64(L == 0) : hi_smem_f32(L == 0)) : 0});
         size_t e = k;
         while (e < par.size() && par[e].first == par[k].first) ++e;
@@ -580,7 +611,14 @@ bd_status plan(bd_ctx* ctx)
         k = e;
     }
     for (ParClass& pc : ctx->par_classes) {
-        const int per_cta = pc.hi ? 1 : pc.threads / 32;
+        const int per_cta = pc.hi || pc.block ? 1 : pc.threads / 32;
+        if (pc.block) {
+            const cudaError_t e = ctx->f64 ? parent_block_smem_f64(pc.L, &pc.smem) : parent_block_smem_f32(pc.L, &pc.smem);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                return fail(ctx, BD_E_CUDA, "parent kernel of tile %d: %s", pc.L, cudaGetErrorString(e));
+            }
+        }
         pc.grid = (pc.warp_count + per_cta - 1) / per_cta;
     }
     // snapshot chunk: up to 64 windows, capped at ~512 MB
@@ -734,7 +772,7 @@ cudaKernelNodeParams parent_node(const bd_ctx* ctx, size_t k, StepParams* pk, vo
     if (pc.hi)
         kp.func = const_cast<void*>(ctx->f64 ? hi_parent_func_f64(pc.L == 0) : hi_parent_func_f32(pc.L == 0));
     else
-        kp.func = const_cast<void*>(ctx->f64 ? parent_func_f64(pc.L, pc.lj) : parent_func_f32(pc.L, pc.lj));
+        kp.func = const_cast<void*>(ctx->f64 ? parent_func_f64(pc.L, pc.lj, pc.block) : parent_func_f32(pc.L, pc.lj, pc.block));
     kp.gridDim = dim3(pc.grid);
     kp.blockDim = dim3(pc.threads);
     kp.sharedMemBytes = (unsigned)pc.smem;

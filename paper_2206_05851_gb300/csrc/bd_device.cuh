@@ -54,6 +54,9 @@ struct ItemDev {
 // Threads of every parent-kernel CTA and of every adjoint-kernel CTA (the
 // kernels size their shared tables by them).
 constexpr int kParentThreads = 64;
+// ... of a CTA of the parent kernel for few parents: one integrating warp,
+// three that draw its noise and sample it.
+constexpr int kParentThreads2 = 128;
 // Replica bonds of a warp per spring of its tile (conf_scratch): 32 lanes of
 // one replica, or of two.
 constexpr int kConfSlots = 64;

@@ -63,8 +63,12 @@ size_t noise_ang_bytes();
 cudaError_t run_noise_tables(void* rad, void* ang, cudaStream_t st);
 
 // Parent kernels per tile; lj: the collapsed-chain step.
-const void* parent_func_f32(int L, bool lj);
-const void* parent_func_f64(int L, bool lj);
+// block: the kernel for few parents (kParentThreads2 threads a warp of
+// parents; in float64 also tile 1).
+const void* parent_func_f32(int L, bool lj, bool block);
+const void* parent_func_f64(int L, bool lj, bool block);
+cudaError_t parent_block_smem_f32(int L, size_t* bytes);
+cudaError_t parent_block_smem_f64(int L, size_t* bytes);
 const void* persist_plain_f32(int variant);     // without the Eq. 5 diagnostics
 const void* persist_plain_f64(int variant);
 const void* persist_conf_f32(int variant);      // with them (bd_window_f32c.cu)

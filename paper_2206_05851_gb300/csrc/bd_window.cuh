@@ -181,6 +181,283 @@ __device__ __forceinline__ void run_one_item(const ItemDev& it, const StepRange&
 }
 
 // ---------------------------------------------------------------------------
+// Few parents of Hooke and FENE chains. CTA g holds parent_warps[g].count parents
+// (chains parent_items[first + s]), each on G lanes of warp 0.
+//
+// A parent's steps are a serial chain, and the one warp of parent_kernel that
+// draws the noise, takes the step and samples it issues about 620
+// instructions a step (4-spring tile) at the rate of a lone warp: 1.1-1.3 us
+// a step in float32, 4.8 us in float64. Only the forces and the update depend on the
+// state, so the rest moves to the CTA's other warps, B steps at a time: warp
+// 0 takes the steps of block k from the noise in shared memory and leaves the
+// bonds of every step there, while warps 1..3 draw the noise of block k + 1
+// and sample the bonds of block k - 1 (TSF sums, ISF criteria; the springs
+// of a helper thread stay with it, so every sum keeps its order). One CTA
+// barrier a block. The rounding sequence is that of step_bonds: the helpers
+// store the difference of the two beads' normals that the update would form.
+// It issues more in all (idle helper lanes, the buffers), so many parents,
+// which fill the GPU anyway, stay with parent_kernel (bd_api.cu:
+// kParentBlockWarps).
+// ---------------------------------------------------------------------------
+template <typename T, int L> struct ParentBlock {
+    static constexpr int helpers = kParentThreads2 - 32;
+    static constexpr int E = 32 * L;                            // springs (and beads) of the CTA
+    static constexpr int B = L <= 4 ? 8 : L <= 7 ? 4 : L <= 10 ? 3 : 2;   // steps a block (48 KB of buffers in float32)
+    static constexpr int NS = (E + helpers - 1) / helpers;      // springs a helper samples
+    static constexpr int rows = 2 * B * 3;                      // rows of E values of each buffer
+    struct Chain {                                              // sampling constants of one parent
+        T H, Hinvb, smin, fc;
+        BellConst bell;
+        int64_t spr_off;
+        int32_t nb, pad;
+    };
+    static constexpr size_t bytes = sizeof(uint4) * E + sizeof(Chain) * 32 + sizeof(T) * 2 * rows * E;
+};
+
+// A lane's L values of a row (value lane L + j), in the widest loads that L allows.
+template <typename T, int L>
+__device__ __forceinline__ void row_load(const T* row, int lane, T (&v)[L])
+{
+    constexpr int W = sizeof(T) == 4 ? (L % 4 == 0 ? 4 : L % 2 == 0 ? 2 : 1) : (L % 2 == 0 ? 2 : 1);
+    struct alignas(sizeof(T) * W) Vec { T e[W]; };
+    const Vec* src = reinterpret_cast<const Vec*>(row + lane * L);
+#pragma unroll
+    for (int j = 0; j < L / W; ++j) {
+        const Vec x = src[j];
+#pragma unroll
+        for (int e = 0; e < W; ++e) v[W * j + e] = x.e[e];
+    }
+}
+template <typename T, int L>
+__device__ __forceinline__ void row_store(T* row, int lane, const T (&v)[L])
+{
+    constexpr int W = sizeof(T) == 4 ? (L % 4 == 0 ? 4 : L % 2 == 0 ? 2 : 1) : (L % 2 == 0 ? 2 : 1);
+    struct alignas(sizeof(T) * W) Vec { T e[W]; };
+    Vec* dst = reinterpret_cast<Vec*>(row + lane * L);
+#pragma unroll
+    for (int j = 0; j < L / W; ++j) {
+        Vec x;
+#pragma unroll
+        for (int e = 0; e < W; ++e) x.e[e] = v[W * j + e];
+        dst[j] = x;
+    }
+}
+
+// step_bonds with the noise differences xi_{i+1} - xi_i of the lane's springs
+// given (the same rounding sequence).
+template <typename T, int L, bool FAST>
+__device__ __forceinline__ int step_bonds_given(T (&qx)[L], T (&qy)[L], T (&qz)[L], const T (&dx)[L],
+                                                const T (&dy)[L], const T (&dz)[L], const LaneCtx& lc,
+                                                const StepConst<T, FAST>& k)
+{
+    int fl = 0;
+    T fx[L], fy[L], fz[L];
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+        const T c = spring_coef<T, FAST>(qx[j], qy[j], qz[j], k.H, k.Hinvb, k.smin, fl);
+        fx[j] = c * qx[j]; fy[j] = c * qy[j]; fz[j] = c * qz[j];
+    }
+    T fmx = shfl(fx[L - 1], lc.src_prev), fmy = shfl(fy[L - 1], lc.src_prev), fmz = shfl(fz[L - 1], lc.src_prev);
+    T fnx = shfl(fx[0], lc.src_next), fny = shfl(fy[0], lc.src_next), fnz = shfl(fz[0], lc.src_next);
+    if (!lc.has_prev) { fmx = T(0); fmy = T(0); fmz = T(0); }
+    if (!lc.has_next) { fnx = T(0); fny = T(0); fnz = T(0); }
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+        const T px = j + 1 < L ? fx[j + 1 < L ? j + 1 : 0] : fnx;
+        const T py = j + 1 < L ? fy[j + 1 < L ? j + 1 : 0] : fny;
+        const T pz = j + 1 < L ? fz[j + 1 < L ? j + 1 : 0] : fnz;
+        if (j < lc.nv) {
+            const T lx = fma(T(-2), fx[j], px + fmx);
+            const T ly = fma(T(-2), fy[j], py + fmy);
+            const T lz = fma(T(-2), fz[j], pz + fmz);
+            const T ox = qx[j], oy = qy[j], oz = qz[j];
+            qx[j] = fma(k.cn, dx[j], fma(k.cd, lx, fma(k.axz, oz, fma(k.axx, ox, ox))));
+            qy[j] = fma(k.cn, dy[j], fma(k.cd, ly, fma(k.ayy, oy, oy)));
+            qz[j] = fma(k.cn, dz[j], fma(k.cd, lz, fma(k.azz, oz, oz)));
+        }
+        fmx = fx[j]; fmy = fy[j]; fmz = fz[j];
+    }
+    return lc.active ? fl : 0;
+}
+
+// The CTA's barrier between blocks, met by its warps in different code.
+__device__ __forceinline__ void parent_barrier()
+{
+    asm volatile("bar.sync 1, %0;" :: "n"(kParentThreads2) : "memory");
+}
+
+template <typename T, int L, bool FAST>
+__global__ void __launch_bounds__(kParentThreads2)
+parent_block_kernel(const StepParams p)
+{
+    using PB = ParentBlock<T, L>;
+    constexpr int E = PB::E, B = PB::B, NS = PB::NS;
+    extern __shared__ uint4 bd_parent_smem[];
+    uint4* ptab = bd_parent_smem;                                        // Philox bead parts, parent s at [s G L, (s + 1) G L)
+    T* noise = reinterpret_cast<T*>(ptab + E);                           // [2][B][3][E]
+    T* bonds = noise + PB::rows * E;                                     // [2][B][3][E]
+    typename PB::Chain* pc = reinterpret_cast<typename PB::Chain*>(bonds + PB::rows * E);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const ParentWarp pw = p.parent_warps[blockIdx.x];
+    const int G = pw.G, P = 32 / G, GL = G * L, beads = P * GL;
+    const int64_t M = p.M;
+    for (int e = threadIdx.x; e < beads; e += blockDim.x) {
+        const int s = e / GL;
+        const int c = p.parent_items[pw.first + min(s, pw.count - 1)];
+        ptab[e] = PhiloxSplit::bead_part((uint32_t)(e - s * GL), (uint32_t)c + p.chain_base, p.rk0, p.rk1);
+    }
+    if ((int)threadIdx.x < pw.count) {
+        const ChainDev& ch = p.chains[p.parent_items[pw.first + threadIdx.x]];
+        StepConst<T, FAST> k;
+        k.load(ch, p);
+        typename PB::Chain& o = pc[threadIdx.x];
+        o.H = k.H; o.Hinvb = k.Hinvb; o.smin = k.smin;
+        o.fc = (T)ch.f_c;
+        o.bell.load(ch.k0, p.dt, ch.dx);
+        o.spr_off = ch.spr_off;
+        o.nb = ch.N - 1;
+    }
+    __syncthreads();
+
+    const int64_t nblk = (p.n_steps + B - 1) / B;
+    if (warp == 0) {
+        // the integrator: wait for the noise of block k, take its steps
+        const int sw = lane / G;
+        const bool active = sw < P && sw < pw.count;
+        const int c = p.parent_items[pw.first + (active ? sw : 0)];
+        const ChainDev& ch = p.chains[c];
+        const int64_t spr_off = ch.spr_off;
+        const LaneCtx lc = make_lane(sw < P ? lane - sw * G : 0, G, L, lane, ch.N - 1, active, 0u, (uint32_t)c + p.chain_base);
+        StepConst<T, FAST> k;
+        k.load(ch, p);
+        T* state = reinterpret_cast<T*>(p.state) + ch.state_off * 3;
+        T* snap = reinterpret_cast<T*>(p.snap);
+        T qx[L], qy[L], qz[L];
+        load_bonds<T, L>(qx, qy, qz, state, lc);
+        int floored = 0;
+        int s_in = (int)(p.t0 % p.S);
+        int64_t w = p.t0 / p.S, left = p.n_steps;
+        for (int64_t b = 0; b <= nblk; ++b) {
+            parent_barrier();
+            const int nb_steps = left < B ? (int)left : B;
+            left -= nb_steps;
+            T* nrow = noise + (b & 1) * (B * 3 * E);
+            T* brow = bonds + (b & 1) * (B * 3 * E);
+#pragma unroll 1
+            for (int s = 0; s < nb_steps; ++s, nrow += 3 * E, brow += 3 * E) {
+                if (s_in == 0)   // the conformation the replicas of window w start from
+                    store_bonds<T, L>(qx, qy, qz, snap + ((w % p.win_ring) * M + spr_off) * 3, lc);
+                T dx[L], dy[L], dz[L];
+                row_load<T, L>(nrow, lane, dx);
+                row_load<T, L>(nrow + E, lane, dy);
+                row_load<T, L>(nrow + 2 * E, lane, dz);
+                floored += step_bonds_given<T, L, FAST>(qx, qy, qz, dx, dy, dz, lc, k);
+                row_store<T, L>(brow, lane, qx);
+                row_store<T, L>(brow + E, lane, qy);
+                row_store<T, L>(brow + 2 * E, lane, qz);
+                if (++s_in == p.S) { s_in = 0; ++w; }
+            }
+        }
+        store_bonds<T, L>(qx, qy, qz, state, lc);
+        if (floored) atomicAdd(p.overext + c, (unsigned long long)floored);
+        return;
+    }
+
+    // helpers: noise of the block ahead, samples of the block behind. A
+    // noise unit is one step of 31 springs (32 beads); a helper thread samples
+    // springs h + 96 j of the CTA.
+    const int h = (int)threadIdx.x - 32;
+    const bool isf_thr = (p.thr_mask & BD_CRIT_ISF) != 0;
+    const bool isf_bell = (p.bell_mask & BD_CRIT_ISF) != 0;
+    ParentSums<T> sums[NS];
+    uint32_t mine = 0, thr_done = 0, bell_done = 0;
+    int par[NS];
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+        const int e = h + PB::helpers * j, s = e / GL;
+        const bool v = s < P && s < pw.count && e - s * GL < pc[s < pw.count ? s : 0].nb;
+        par[j] = v ? s : 0;
+        const int64_t m = v ? pc[s].spr_off + (e - s * GL) : 0;
+        sums[j].start(v ? p.tsf_acc[m] : 0.0, v ? p.exp1[CRIT_Q_ISF * M + m] - p.lam[CRIT_Q_ISF * M + m] : 0.0);
+        if (v) mine |= 1u << j;
+        if (!v || p.first_thr[CRIT_Q_ISF * M + m] >= 0) thr_done |= 1u << j;
+        if (!v || p.first_bell[CRIT_Q_ISF * M + m] >= 0) bell_done |= 1u << j;
+    }
+    const int chunks = (beads + 30) / 31;
+    int s_in = (int)(p.t0 % p.S);
+    int64_t w = p.t0 / p.S;
+    for (int64_t b = -1; b <= nblk; ++b) {
+        if (b + 1 < nblk) {                                     // noise of block b + 1
+            const int64_t t_b = p.t0 + (b + 1) * B;
+            const int steps = p.t0 + p.n_steps - t_b < B ? (int)(p.t0 + p.n_steps - t_b) : B;
+            T* nb0 = noise + ((b + 1) & 1) * (B * 3 * E);
+            for (int u = warp - 1; u < steps * chunks; u += PB::helpers / 32) {
+                const int s = u / chunks, e = (u - s * chunks) * 31 + lane;
+                const uint3 sp = PhiloxSplit::step_part((uint32_t)(t_b + s), noise_word(0u), p.rk0);
+                T z0, z1, z2;
+                bead_noise_split<T, FAST, 0>(ptab[min(e, beads - 1)], sp, p, 0u, z0, z1, z2);
+                const T y0 = __shfl_down_sync(0xffffffffu, z0, 1), y1 = __shfl_down_sync(0xffffffffu, z1, 1),
+                        y2 = __shfl_down_sync(0xffffffffu, z2, 1);
+                if (lane < 31 && e < beads) {
+                    T* row = nb0 + s * 3 * E + e;
+                    row[0] = y0 - z0;
+                    row[E] = y1 - z1;
+                    row[2 * E] = y2 - z2;
+                }
+            }
+        }
+        if (b >= 1) {                                           // samples of block b - 1
+            const int64_t t_b = p.t0 + (b - 1) * B;
+            const int steps = p.t0 + p.n_steps - t_b < B ? (int)(p.t0 + p.n_steps - t_b) : B;
+            const T* brow = bonds + ((b - 1) & 1) * (B * 3 * E) + h;
+#pragma unroll 1
+            for (int s = 0; s < steps; ++s, brow += 3 * E) {
+                const bool ends = ++s_in == p.S;
+#pragma unroll
+                for (int j = 0; j < NS; ++j) {
+                    if (!(mine & (1u << j))) continue;
+                    const typename PB::Chain& o = pc[par[j]];
+                    const int d = PB::helpers * j;
+                    const T f = spring_tension<T, FAST>(brow[d], brow[E + d], brow[2 * E + d], o.H, o.Hinvb, o.smin);
+                    sums[j].add_isf(f);
+                    const int64_t m = o.spr_off + (h + d - par[j] * GL);
+                    if (isf_thr && !(thr_done & (1u << j)) && f >= o.fc) {
+                        thr_done |= 1u << j;
+                        p.first_thr[CRIT_Q_ISF * M + m] = t_b + s + 1;
+                    }
+                    if (isf_bell) {
+                        const bool reached = sums[j].add_hazard(f, o.bell, p.lam + CRIT_Q_ISF * M + m);
+                        if (!(bell_done & (1u << j)) && reached) {
+                            bell_done |= 1u << j;
+                            p.first_bell[CRIT_Q_ISF * M + m] = t_b + s + 1;
+                        }
+                    }
+                    if (ends) {
+                        p.tsf_hist[w * M + m] = sums[j].tsf_sum() / (double)p.S;
+                        double rem = 0.0;
+                        if (isf_bell) {
+                            const double lam = p.lam[CRIT_Q_ISF * M + m] + sums[j].hazard();
+                            p.lam[CRIT_Q_ISF * M + m] = lam;
+                            rem = p.exp1[CRIT_Q_ISF * M + m] - lam;
+                        }
+                        sums[j].next_window(rem);
+                    }
+                }
+                if (ends) { s_in = 0; ++w; }
+            }
+        }
+        if (b < nblk) parent_barrier();
+    }
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+        if (!(mine & (1u << j))) continue;
+        const int64_t m = pc[par[j]].spr_off + (h + PB::helpers * j - par[j] * GL);
+        p.tsf_acc[m] = sums[j].tsf_sum();
+        if (isf_bell) p.lam[CRIT_Q_ISF * M + m] += sums[j].hazard();
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Parents. Global warp g holds parent_warps[g].count parents (chains
 // parent_items[first + s]), each on G lanes.
 // Per step: update, then sample the parent's spring forces (ISF): TSF window

@@ -8,22 +8,37 @@
 namespace bdra {
 
 namespace {
-template <int L> const void* parent_fn(bool lj)
+template <int L> const void* parent_fn(bool lj, bool block)
 {
-    return lj ? (const void*)parent_kernel<double, L, false, true> : (const void*)parent_kernel<double, L, false, false>;
+    if (block) return (const void*)parent_block_kernel<double, L, false>;
+    if constexpr (L == 1) return nullptr;        // a tile of the block kernel only
+    else return lj ? (const void*)parent_kernel<double, L, false, true> : (const void*)parent_kernel<double, L, false, false>;
 }
 }  // namespace
 
-#define BD_PARENT_TILES(X) X(2) X(4) X(7) X(10) X(13) X(16)
+#define BD_PARENT_TILES(X) X(1) X(2) X(4) X(7) X(10) X(13) X(16)
 
-const void* parent_func_f64(int L, bool lj)
+const void* parent_func_f64(int L, bool lj, bool block)
 {
     switch (L) {
-#define X(l) case l: return parent_fn<l>(lj);
+#define X(l) case l: return parent_fn<l>(lj, block);
         BD_PARENT_TILES(X)
 #undef X
     default: return nullptr;
     }
+}
+
+// Dynamic shared memory of a block-kernel CTA, allowed here for the current device.
+cudaError_t parent_block_smem_f64(int L, size_t* bytes)
+{
+    *bytes = 0;
+    switch (L) {
+#define X(l) case l: *bytes = ParentBlock<double, l>::bytes; break;
+        BD_PARENT_TILES(X)
+#undef X
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaFuncSetAttribute(parent_func_f64(L, false, true), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*bytes);
 }
 
 const void* persist_plain_f64(int v)
