@@ -296,9 +296,11 @@ bd_status bd_get_plan(bd_ctx* ctx, int32_t* variant, int32_t* groups, double* co
 
 /* Kernel timing for measurement tools. Each chunk graph that bd_step launches
  * records CUDA events before its parent kernels, between the parent and
- * replica kernels, and after the replica kernels. enable != 0: after every
- * chunk bd_step waits for those events and accumulates the two intervals
- * (enable = 0 stops; bd_step then never waits). bd_kernel_times
+ * replica kernels, and after the replica kernels. enable != 0: every chunk
+ * runs its parents before its replicas (small batches and chains with
+ * hydrodynamic interaction otherwise overlap the two; the results are the
+ * same), and bd_step waits for those events after it and accumulates the two
+ * intervals (enable = 0 stops; bd_step then never waits). bd_kernel_times
  * synchronises the stream, returns the accumulated device time in
  * milliseconds and the launch counts since the last call (index 0: parent
  * kernels, 1: replica kernels) and resets them. ms and launches are host

@@ -24,7 +24,7 @@ struct VarClass {      // one persistent replica launch: the work items of one s
     int item_begin, item_count;
     int threads;
     int resident;      // CTAs of this kernel that the GPU holds
-    int grid, grid_y, block;   // this chunk's CTAs and their threads (chunk_shapes)
+    struct { int grid, grid_y, block; } shape[2];   // CTAs and threads of the chunk's two launches (chunk_shapes)
     size_t smem;       // dynamic shared memory per CTA
     size_t conf_off;   // its warps' part of the Eq. 5 scratch (elements)
 };
@@ -85,7 +85,7 @@ struct bd_ctx {
     double* d_dbead = nullptr;          // [max_windows][sum N][3]
     double* d_rgz = nullptr;            // [max_windows][n_chains]
     void* d_conf_scratch = nullptr;     // window-end bonds of the resident warps
-    size_t conf_elems = 0;
+    size_t conf_elems = 0;              // of one replica launch; the two of a chunk may overlap
     double* d_tsf = nullptr;
     double* d_tsf_acc = nullptr;
     double* d_lam = nullptr;
@@ -98,12 +98,14 @@ struct bd_ctx {
     const void* noise_rad = nullptr;    // the device's float64 noise tables (float64 contexts; shared)
     const void* noise_ang = nullptr;
     int32_t* d_queue = nullptr;         // per variant launch queue_len() work-item counters, one a part
-    // the step chunk as a CUDA graph: queue reset, parent kernels, one
-    // persistent replica kernel per variant (parallel branches), and three
-    // event records (start, after the parents, after the replicas)
+    // the step chunk as a CUDA graph (build_graph): queue reset, the parent
+    // kernels and the persistent replica kernels (one per variant) in two
+    // stages each, three event records (start, after the first parents, after
+    // the replicas) and the window fold
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
-    std::vector<cudaGraphNode_t> par_nodes, rep_nodes;
+    std::vector<cudaGraphNode_t> par_nodes[2], rep_nodes[2];
+    bool par_on[2] = {true, true}, rep_on[2] = {true, true};   // which stages' nodes are enabled
     cudaGraphNode_t ev_nodes[3] = {nullptr, nullptr, nullptr};
     cudaGraphNode_t fold_node = nullptr;     // partial sums -> RSF history, after the replicas
     cudaEvent_t idle_ev[3] = {nullptr, nullptr, nullptr};
@@ -539,7 +541,7 @@ bd_status plan(bd_ctx* ctx)
     const int threads = ctx->f64 ? persist_threads_f64() : persist_threads_f32();
     for (size_t k = 0; k < items.size(); ++k) {
         if (ctx->var_classes.empty() || ctx->var_classes.back().variant != items[k].variant)
-            ctx->var_classes.push_back(VarClass{items[k].variant, (int)k, 0, threads, 0, 0, 1, 0, 0, 0});
+            ctx->var_classes.push_back(VarClass{items[k].variant, (int)k, 0, threads, 0, {}, 0, 0});
         ctx->var_classes.back().item_count++;
     }
     ctx->conf_elems = 0;
@@ -685,9 +687,8 @@ int replica_parts(int64_t items, int64_t places, int64_t W, int64_t per_place)
     return (int)std::max<int64_t>(1, std::min(W, (per_place * places + items - 1) / items));
 }
 
-// Work-item counters of one replica launch: a chunk touches at most
-// chunk_windows + 1 windows, so it has at most that many parts.
-int64_t queue_len(const bd_ctx* ctx) { return ctx->chunk_windows + 1; }
+// Work-item counters of one replica launch, one a part.
+int64_t queue_len(const bd_ctx* ctx) { return ctx->chunk_windows; }
 
 // Splits every replica launch of steps [t0, t0 + n) and sizes its grid. A
 // launch with more units than the GPU holds warps takes every SM and goes
@@ -696,7 +697,7 @@ int64_t queue_len(const bd_ctx* ctx) { return ctx->chunk_windows + 1; }
 // part with CTAs of its own that hold as few warps as that share allows: a
 // warp alone on its SM sub-partition steps fastest (the float64 chain of 20
 // beads: 1.2 ms for ten windows side by side, 18.7 ms one after another).
-void chunk_shapes(bd_ctx* ctx, int64_t t0, int64_t n, std::vector<StepParams>& rp)
+void chunk_shapes(bd_ctx* ctx, int stage, int64_t t0, int64_t n, std::vector<StepParams>& rp)
 {
     const int64_t S = ctx->cfg.window_steps;
     const int64_t W = std::max<int64_t>(1, (t0 + n + S - 1) / S - t0 / S);
@@ -712,9 +713,7 @@ void chunk_shapes(bd_ctx* ctx, int64_t t0, int64_t n, std::vector<StepParams>& r
         rp[k].win_per_part = (int32_t)((W + parts - 1) / parts);
         rp[k].n_parts = (int32_t)((W + rp[k].win_per_part - 1) / rp[k].win_per_part);
         if (hi) {
-            vc.grid = rp[k].n_parts * vc.item_count;
-            vc.grid_y = 1;
-            vc.block = vc.threads;
+            vc.shape[stage] = {rp[k].n_parts * vc.item_count, 1, vc.threads};
             continue;
         }
         total_units += (int64_t)rp[k].n_parts * vc.item_count;
@@ -729,39 +728,82 @@ void chunk_shapes(bd_ctx* ctx, int64_t t0, int64_t n, std::vector<StepParams>& r
         int64_t warps = std::max<int64_t>(1, (units + ctas - 1) / ctas);
         while (warps <= most && (vc.item_count + warps - 1) / warps * parts > ctas) ++warps;
         if (warps <= most) {              // one unit a warp, every part its own CTAs
-            vc.grid_y = (int)parts;
-            vc.grid = (int)((vc.item_count + warps - 1) / warps);
-            vc.block = (int)(32 * warps);
+            vc.shape[stage] = {(int)((vc.item_count + warps - 1) / warps), (int)parts, (int)(32 * warps)};
         } else {
-            vc.grid_y = 1;
-            vc.grid = (int)std::min<int64_t>((units + most - 1) / most, vc.resident);
-            vc.block = vc.threads;
+            vc.shape[stage] = {(int)std::min<int64_t>((units + most - 1) / most, vc.resident), 1, vc.threads};
         }
     }
 }
 
-// Kernel-node parameters of the chunk graph for one chunk [t0, t0 + n).
-// `pp` / `rp` hold one StepParams per node (kernelParams point into them).
-void chunk_params(bd_ctx* ctx, int64_t t0, int64_t n, std::vector<StepParams>& pp,
-                  std::vector<StepParams>& rp)
+// One chunk as up to two parent and two replica launches.
+struct Stage { int64_t t0, n; bool on, store; };
+struct ChunkStages { Stage par[2], rep[2]; };
+
+// The replicas of a window need the parent only up to its start, so a
+// chunk's first window runs beside the parents' way through all windows but
+// the last, and the other windows beside the parents' last one:
+//   rep[0]: first window     | rep[1]: the rest, after par[0]
+//   par[0]: all but the last | par[1]: the last, after par[0]
+// That is for launches that leave room (at most half the warps) and for
+// chains with hydrodynamic interaction (a CTA a slot, many per SM). A
+// free-draining launch that fills the GPU holds every register of it, so there
+// the parents go first (par[0], rep[1]); so they do while the two are timed
+// apart, and where the chunk starts inside a window (bd_step ends such a chunk
+// with that window).
+ChunkStages chunk_stages(const bd_ctx* ctx, int64_t t0, int64_t n)
+{
+    const int64_t S = ctx->cfg.window_steps, W = (n + S - 1) / S;
+    int64_t items = 0, places = 0;
+    bool hi = false;
+    for (const VarClass& vc : ctx->var_classes) {
+        if (variant_hi(vc.variant)) { hi = true; continue; }
+        items += vc.item_count;
+        places = std::max<int64_t>(places, (int64_t)vc.resident * (vc.threads / 32));
+    }
+    ChunkStages c;
+    if (ctx->timing || t0 % S != 0 || !(hi || 2 * items <= places)) {
+        c.par[0] = {t0, n, true, true};
+        c.par[1] = {t0, 0, false, false};
+        c.rep[0] = {t0, 0, false, false};
+        c.rep[1] = {t0, n, true, true};
+        return c;
+    }
+    const int64_t first = std::min(n, S), ahead = (W - 1) * S;
+    c.par[0] = {t0, ahead, ahead > 0, false};
+    c.par[1] = {t0 + ahead, n - ahead, true, true};
+    c.rep[0] = {t0, first, true, W == 1};
+    c.rep[1] = {t0 + first, n - first, n > first, true};
+    return c;
+}
+
+// Kernel-node parameters of one stage of a chunk's graph. `pp` / `rp` hold one
+// StepParams per node (kernelParams point into them).
+void parent_params(const bd_ctx* ctx, const Stage& st, std::vector<StepParams>& pp)
 {
     StepParams p = base_params(ctx);
-    p.t0 = t0; p.n_steps = n;
+    p.t0 = st.t0; p.n_steps = st.n;
+    p.store_state = st.store;
     pp.assign(ctx->par_classes.size(), p);
     for (size_t k = 0; k < ctx->par_classes.size(); ++k) {
         const ParClass& pc = ctx->par_classes[k];
         pp[k].parent_warps = ctx->d_parent_warps + pc.warp_begin;
         pp[k].n_parent_warps = pc.warp_count;
     }
+}
+void replica_params(bd_ctx* ctx, int stage, const Stage& st, std::vector<StepParams>& rp)
+{
+    StepParams p = base_params(ctx);
+    p.t0 = st.t0; p.n_steps = st.n;
+    p.store_state = st.store;
     rp.assign(ctx->var_classes.size(), p);
     for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
         const VarClass& vc = ctx->var_classes[k];
         rp[k].items = ctx->d_items + vc.item_begin;
         rp[k].n_items = vc.item_count;
-        rp[k].queue = ctx->d_queue + k * queue_len(ctx);
-        if (ctx->conf) rp[k].conf_scratch = (char*)ctx->d_conf_scratch + vc.conf_off * ctx->tsize;
+        rp[k].queue = ctx->d_queue + (stage * ctx->var_classes.size() + k) * queue_len(ctx);
+        if (ctx->conf) rp[k].conf_scratch = (char*)ctx->d_conf_scratch + (stage * ctx->conf_elems + vc.conf_off) * ctx->tsize;
     }
-    chunk_shapes(ctx, t0, n, rp);
+    chunk_shapes(ctx, stage, st.t0, st.n, rp);
 }
 
 cudaKernelNodeParams parent_node(const bd_ctx* ctx, size_t k, StepParams* pk, void** args)
@@ -780,7 +822,7 @@ cudaKernelNodeParams parent_node(const bd_ctx* ctx, size_t k, StepParams* pk, vo
     return kp;
 }
 
-cudaKernelNodeParams replica_node(const bd_ctx* ctx, size_t k, StepParams* rk, void** args)
+cudaKernelNodeParams replica_node(const bd_ctx* ctx, int stage, size_t k, StepParams* rk, void** args)
 {
     const VarClass& vc = ctx->var_classes[k];
     args[0] = rk;
@@ -791,8 +833,8 @@ cudaKernelNodeParams replica_node(const bd_ctx* ctx, size_t k, StepParams* rk, v
     else
         kp.func = const_cast<void*>(ctx->f64 ? persist_func_f64(vc.variant, ctx->conf)
                                              : persist_func_f32(vc.variant, ctx->conf));
-    kp.gridDim = dim3(vc.grid, vc.grid_y);
-    kp.blockDim = dim3(vc.block);
+    kp.gridDim = dim3(vc.shape[stage].grid, vc.shape[stage].grid_y);
+    kp.blockDim = dim3(vc.shape[stage].block);
     kp.sharedMemBytes = (unsigned)vc.smem;
     kp.kernelParams = args;
     return kp;
@@ -835,14 +877,21 @@ void drop_graph(bd_ctx* ctx)
     if (ctx->graph) cudaGraphDestroy(ctx->graph);
     ctx->gexec = nullptr;
     ctx->graph = nullptr;
-    ctx->par_nodes.clear();
-    ctx->rep_nodes.clear();
+    for (int j = 0; j < 2; ++j) {
+        ctx->par_nodes[j].clear();
+        ctx->rep_nodes[j].clear();
+        ctx->par_on[j] = ctx->rep_on[j] = true;
+    }
     cudaGetLastError();
 }
 
-// Builds the chunk graph: start event -> queue reset -> parent kernels (one
-// per tile, parallel) -> mid event -> replica kernels (one per variant,
-// parallel) -> end event.
+// Builds the chunk graph (nodes of one kind are parallel branches):
+//   start event -> queue reset -> par[0] -> mid event -> par[1]
+//                             |                       -> rep[1] -+-> end event -> fold
+//                             +-> rep[0] ------------------------+
+// A chunk enables the stages it has (chunk_stages). The parents' nodes have
+// the higher priority: their CTAs take the first free places, so the next
+// stage is not held up behind the queue of replica CTAs.
 bd_status build_graph(bd_ctx* ctx)
 {
     drop_graph(ctx);
@@ -850,37 +899,55 @@ bd_status build_graph(bd_ctx* ctx)
         if (!ctx->idle_ev[i]) BD_CUDA(ctx, cudaEventCreate(&ctx->idle_ev[i]));
     BD_CUDA(ctx, cudaGraphCreate(&ctx->graph, 0));
     std::vector<StepParams> pp, rp;
-    chunk_params(ctx, 0, 0, pp, rp);
-    cudaGraphNode_t prev;
+    const Stage whole = {0, 1, true, true};
+    parent_params(ctx, whole, pp);
     BD_CUDA(ctx, cudaGraphAddEventRecordNode(&ctx->ev_nodes[0], ctx->graph, nullptr, 0, ctx->idle_ev[0]));
     cudaMemsetParams ms = {};
     ms.dst = ctx->d_queue;
     ms.value = 0;
     ms.elementSize = sizeof(int32_t);
-    ms.width = ctx->var_classes.size() * queue_len(ctx);
+    ms.width = 2 * ctx->var_classes.size() * queue_len(ctx);
     ms.height = 1;
     ms.pitch = 0;
-    cudaGraphNode_t mnode;
-    BD_CUDA(ctx, cudaGraphAddMemsetNode(&mnode, ctx->graph, &ctx->ev_nodes[0], 1, &ms));
-    prev = mnode;
-    for (size_t k = 0; k < ctx->par_classes.size(); ++k) {      // parallel branches
-        void* args[1];
-        cudaKernelNodeParams kp = parent_node(ctx, k, &pp[k], args);
-        cudaGraphNode_t nd;
-        BD_CUDA(ctx, cudaGraphAddKernelNode(&nd, ctx->graph, &prev, 1, &kp));
-        ctx->par_nodes.push_back(nd);
-    }
-    BD_CUDA(ctx, cudaGraphAddEventRecordNode(&ctx->ev_nodes[1], ctx->graph, ctx->par_nodes.data(),
-                                             ctx->par_nodes.size(), ctx->idle_ev[1]));
-    for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
-        void* args[1];
-        cudaKernelNodeParams kp = replica_node(ctx, k, &rp[k], args);
-        cudaGraphNode_t nd;
-        BD_CUDA(ctx, cudaGraphAddKernelNode(&nd, ctx->graph, &ctx->ev_nodes[1], 1, &kp));
-        ctx->rep_nodes.push_back(nd);
-    }
-    BD_CUDA(ctx, cudaGraphAddEventRecordNode(&ctx->ev_nodes[2], ctx->graph, ctx->rep_nodes.data(),
-                                             ctx->rep_nodes.size(), ctx->idle_ev[2]));
+    cudaGraphNode_t reset;
+    BD_CUDA(ctx, cudaGraphAddMemsetNode(&reset, ctx->graph, &ctx->ev_nodes[0], 1, &ms));
+    int least = 0, greatest = 0;
+    BD_CUDA(ctx, cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    cudaLaunchAttributeValue high = {};
+    high.priority = greatest;
+    auto parents = [&](int j, cudaGraphNode_t after) -> cudaError_t {
+        for (size_t k = 0; k < ctx->par_classes.size(); ++k) {
+            void* args[1];
+            cudaKernelNodeParams kp = parent_node(ctx, k, &pp[k], args);
+            cudaGraphNode_t nd;
+            cudaError_t e = cudaGraphAddKernelNode(&nd, ctx->graph, &after, 1, &kp);
+            if (e == cudaSuccess) e = cudaGraphKernelNodeSetAttribute(nd, cudaLaunchAttributePriority, &high);
+            if (e != cudaSuccess) return e;
+            ctx->par_nodes[j].push_back(nd);
+        }
+        return cudaSuccess;
+    };
+    auto replicas = [&](int j, cudaGraphNode_t after) -> cudaError_t {
+        replica_params(ctx, j, whole, rp);
+        for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
+            void* args[1];
+            cudaKernelNodeParams kp = replica_node(ctx, j, k, &rp[k], args);
+            cudaGraphNode_t nd;
+            const cudaError_t e = cudaGraphAddKernelNode(&nd, ctx->graph, &after, 1, &kp);
+            if (e != cudaSuccess) return e;
+            ctx->rep_nodes[j].push_back(nd);
+        }
+        return cudaSuccess;
+    };
+    BD_CUDA(ctx, parents(0, reset));
+    BD_CUDA(ctx, cudaGraphAddEventRecordNode(&ctx->ev_nodes[1], ctx->graph, ctx->par_nodes[0].data(),
+                                             ctx->par_nodes[0].size(), ctx->idle_ev[1]));
+    BD_CUDA(ctx, parents(1, ctx->ev_nodes[1]));
+    BD_CUDA(ctx, replicas(0, reset));
+    BD_CUDA(ctx, replicas(1, ctx->ev_nodes[1]));
+    std::vector<cudaGraphNode_t> done = ctx->rep_nodes[0];
+    done.insert(done.end(), ctx->rep_nodes[1].begin(), ctx->rep_nodes[1].end());
+    BD_CUDA(ctx, cudaGraphAddEventRecordNode(&ctx->ev_nodes[2], ctx->graph, done.data(), done.size(), ctx->idle_ev[2]));
     {
         FoldParams fp;
         void* args[1];
@@ -888,6 +955,15 @@ bd_status build_graph(bd_ctx* ctx)
         BD_CUDA(ctx, cudaGraphAddKernelNode(&ctx->fold_node, ctx->graph, &ctx->ev_nodes[2], 1, &kp));
     }
     BD_CUDA(ctx, cudaGraphInstantiate(&ctx->gexec, ctx->graph, 0));
+    return BD_OK;
+}
+
+// Enables or disables one stage's nodes in the executable graph.
+bd_status switch_stage(bd_ctx* ctx, const std::vector<cudaGraphNode_t>& nodes, bool& on, bool want)
+{
+    if (on == want) return BD_OK;
+    for (cudaGraphNode_t nd : nodes) BD_CUDA(ctx, cudaGraphNodeSetEnabled(ctx->gexec, nd, want ? 1u : 0u));
+    on = want;
     return BD_OK;
 }
 
@@ -903,7 +979,8 @@ bd_status reset_kinetics(bd_ctx* ctx)
     return BD_OK;
 }
 
-bd_status load_positions(bd_ctx* ctx, const double* pos)
+// The conformations, and the snapshot of the window that starts at `step`.
+bd_status load_positions(bd_ctx* ctx, const double* pos, int64_t step)
 {
     const size_t n = sizeof(double) * 3 * (size_t)ctx->n_beads;
     const double* src = pos;
@@ -915,7 +992,17 @@ bd_status load_positions(bd_ctx* ctx, const double* pos)
     }
     ++ctx->launches;
     BD_CUDA(ctx, run_set_bonds(ctx->f64, ctx->d_chains, ctx->d_spring_chain, ctx->M, src,
-                               ctx->d_state, ctx->stream));
+                               ctx->d_state,
+                               (char*)ctx->d_snap + (step / ctx->cfg.window_steps) % ctx->part_ring * ctx->M * 3 * ctx->tsize,
+                               ctx->stream));
+    for (const ParClass& pc : ctx->par_classes) {
+        if (!pc.hi) continue;
+        StepParams p = base_params(ctx);
+        p.t0 = step;
+        p.parent_warps = ctx->d_parent_warps + pc.warp_begin;
+        ++ctx->launches;
+        BD_CUDA(ctx, ctx->f64 ? run_hi_snap_f64(pc.warp_count, p, ctx->stream) : run_hi_snap_f32(pc.warp_count, p, ctx->stream));
+    }
     if (src != pos) BD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return BD_OK;
 }
@@ -1142,18 +1229,18 @@ bd_status replan(bd_ctx* ctx)
     if ((s = dalloc(ctx, (void**)&ctx->d_part, sizeof(double) * (size_t)ctx->part_ring * (size_t)ctx->part_stride)) != BD_OK)
         return s;
     if (ctx->conf) {
-        dfree(ctx, ctx->d_conf_scratch, std::max<size_t>(ctx->tsize * old_conf, 16));
+        dfree(ctx, ctx->d_conf_scratch, std::max<size_t>(2 * ctx->tsize * old_conf, 16));
         ctx->d_conf_scratch = nullptr;
-        if ((s = dalloc(ctx, &ctx->d_conf_scratch, ctx->tsize * ctx->conf_elems)) != BD_OK) return s;
+        if ((s = dalloc(ctx, &ctx->d_conf_scratch, 2 * ctx->tsize * ctx->conf_elems)) != BD_OK) return s;
         dfree(ctx, ctx->d_dpart, std::max<size_t>(sizeof(double) * 3 * (size_t)ctx->part_ring * (size_t)old_bpart, 16));
         ctx->d_dpart = nullptr;
         if ((s = dalloc(ctx, (void**)&ctx->d_dpart, sizeof(double) * 3 * (size_t)ctx->part_ring *
                                                         (size_t)ctx->bpart_stride)) != BD_OK)
             return s;
     }
-    dfree(ctx, ctx->d_queue, std::max<size_t>(sizeof(int32_t) * queue_len(ctx) * old_queue, 16));
+    dfree(ctx, ctx->d_queue, std::max<size_t>(sizeof(int32_t) * 2 * queue_len(ctx) * old_queue, 16));
     ctx->d_queue = nullptr;
-    if ((s = dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * queue_len(ctx) * ctx->var_classes.size())) != BD_OK) return s;
+    if ((s = dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * 2 * queue_len(ctx) * ctx->var_classes.size())) != BD_OK) return s;
     return build_graph(ctx);
 }
 
@@ -1390,7 +1477,7 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
             BD_TRY(dalloc(ctx, (void**)&ctx->d_dpart, sizeof(double) * 3 * (size_t)ctx->part_ring *
                                                           (size_t)ctx->bpart_stride));
             BD_TRY(dalloc(ctx, (void**)&ctx->d_dbead, sizeof(double) * 3 * (size_t)W * (size_t)ctx->n_beads));
-            BD_TRY(dalloc(ctx, &ctx->d_conf_scratch, ctx->tsize * ctx->conf_elems));
+            BD_TRY(dalloc(ctx, &ctx->d_conf_scratch, 2 * ctx->tsize * ctx->conf_elems));
             BD_TRY(dalloc(ctx, (void**)&ctx->d_rgz, sizeof(double) * (size_t)W * (size_t)C));
         }
         BD_TRY(dalloc(ctx, (void**)&ctx->d_tsf, sizeof(double) * (size_t)W * (size_t)M));
@@ -1407,7 +1494,7 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
             goto failed;
         }
         BD_TRY(dalloc(ctx, (void**)&ctx->d_evt_scratch, sizeof(int64_t) * (size_t)(event_blocks(M) + 2)));
-        BD_TRY(dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * queue_len(ctx) * ctx->var_classes.size()));
+        BD_TRY(dalloc(ctx, (void**)&ctx->d_queue, sizeof(int32_t) * 2 * queue_len(ctx) * ctx->var_classes.size()));
         BD_TRY(build_graph(ctx));
         if (cfg->checkpoint_steps > 0) BD_TRY(adj_plan(ctx));
         {
@@ -1416,7 +1503,7 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
             if (e != cudaSuccess) { cudaGetLastError(); s = fail(ctx, BD_E_CUDA, "exp1: %s", cudaGetErrorString(e)); goto failed; }
         }
         BD_TRY(reset_kinetics(ctx));
-        BD_TRY(load_positions(ctx, init_pos));
+        BD_TRY(load_positions(ctx, init_pos, 0));
         {
             cudaError_t e = cudaStreamSynchronize(ctx->stream);
             if (e != cudaSuccess) { cudaGetLastError(); s = fail(ctx, BD_E_CUDA, "set-up: %s", cudaGetErrorString(e)); goto failed; }
@@ -1460,19 +1547,33 @@ bd_status bd_step(bd_ctx* ctx, int64_t n_steps)
         return fail(ctx, BD_E_CAPACITY, "run to step %lld needs %lld windows; max_windows is %lld",
                     (long long)t_end, (long long)(t_end / S), (long long)ctx->cfg.max_windows);
     std::vector<StepParams> pp, rp;
-    std::vector<void*> pargs(ctx->par_nodes.size()), rargs(ctx->rep_nodes.size());
     int64_t t = ctx->step;
     while (t < t_end) {
+        // a chunk starts at a window start, or lies inside one window
         const int64_t w_first = (t + S - 1) / S;
-        const int64_t chunk_end = std::min(t_end, (w_first + ctx->chunk_windows) * S);
-        chunk_params(ctx, t, chunk_end - t, pp, rp);
-        for (size_t k = 0; k < ctx->par_nodes.size(); ++k) {
-            cudaKernelNodeParams kp = parent_node(ctx, k, &pp[k], &pargs[k]);
-            BD_CUDA(ctx, cudaGraphExecKernelNodeSetParams(ctx->gexec, ctx->par_nodes[k], &kp));
-        }
-        for (size_t k = 0; k < ctx->rep_nodes.size(); ++k) {
-            cudaKernelNodeParams kp = replica_node(ctx, k, &rp[k], &rargs[k]);
-            BD_CUDA(ctx, cudaGraphExecKernelNodeSetParams(ctx->gexec, ctx->rep_nodes[k], &kp));
+        const int64_t chunk_end = std::min(t_end, t % S != 0 ? w_first * S : (w_first + ctx->chunk_windows) * S);
+        const ChunkStages cs = chunk_stages(ctx, t, chunk_end - t);
+        for (int j = 0; j < 2; ++j) {
+            bd_status s = switch_stage(ctx, ctx->par_nodes[j], ctx->par_on[j], cs.par[j].on);
+            if (s == BD_OK) s = switch_stage(ctx, ctx->rep_nodes[j], ctx->rep_on[j], cs.rep[j].on);
+            if (s != BD_OK) return s;
+            void* args[1];
+            if (cs.par[j].on) {
+                parent_params(ctx, cs.par[j], pp);
+                for (size_t k = 0; k < ctx->par_nodes[j].size(); ++k) {
+                    cudaKernelNodeParams kp = parent_node(ctx, k, &pp[k], args);
+                    BD_CUDA(ctx, cudaGraphExecKernelNodeSetParams(ctx->gexec, ctx->par_nodes[j][k], &kp));
+                }
+                ctx->launches += (int64_t)ctx->par_nodes[j].size();
+            }
+            if (cs.rep[j].on) {
+                replica_params(ctx, j, cs.rep[j], rp);
+                for (size_t k = 0; k < ctx->rep_nodes[j].size(); ++k) {
+                    cudaKernelNodeParams kp = replica_node(ctx, j, k, &rp[k], args);
+                    BD_CUDA(ctx, cudaGraphExecKernelNodeSetParams(ctx->gexec, ctx->rep_nodes[j][k], &kp));
+                }
+                ctx->launches += (int64_t)ctx->rep_nodes[j].size();
+            }
         }
         {   // fold the windows this chunk completes, [t / S, chunk_end / S), into the RSF history
             FoldParams fp;
@@ -1481,7 +1582,7 @@ bd_status bd_step(bd_ctx* ctx, int64_t n_steps)
             BD_CUDA(ctx, cudaGraphExecKernelNodeSetParams(ctx->gexec, ctx->fold_node, &kp));
         }
         BD_CUDA(ctx, cudaGraphLaunch(ctx->gexec, ctx->stream));
-        ctx->launches += (int64_t)(ctx->par_nodes.size() + ctx->rep_nodes.size() + 1);
+        ++ctx->launches;
         if (ctx->cfg.checkpoint_steps > 0) {
             bd_status s = keep_checkpoints(ctx, w_first, (chunk_end + S - 1) / S);
             if (s != BD_OK) return s;
@@ -1494,8 +1595,8 @@ bd_status bd_step(bd_ctx* ctx, int64_t n_steps)
             BD_CUDA(ctx, cudaEventElapsedTime(&y, ctx->idle_ev[1], ctx->idle_ev[2]));
             ctx->timed_ms[0] += x;
             ctx->timed_ms[1] += y;
-            ctx->timed_n[0] += (int64_t)ctx->par_nodes.size();
-            ctx->timed_n[1] += (int64_t)ctx->rep_nodes.size();
+            ctx->timed_n[0] += (int64_t)ctx->par_nodes[0].size();
+            ctx->timed_n[1] += (int64_t)ctx->rep_nodes[1].size();
         }
         t = chunk_end;
         ctx->step = t;
@@ -1640,7 +1741,7 @@ bd_status bd_set_positions(bd_ctx* ctx, const double* pos, int64_t step)
         return fail(ctx, BD_E_CAPACITY, "step beyond max_windows");
     bd_status s = reset_kinetics(ctx);
     if (s != BD_OK) return s;
-    s = load_positions(ctx, pos);
+    s = load_positions(ctx, pos, step);
     if (s != BD_OK) return s;
     ctx->step = step;
     ctx->origin = step;

@@ -89,7 +89,8 @@ struct StepParams {
     const ParentWarp* parent_warps;  // parent kernel: warps of this launch
     int32_t n_parent_warps;
     void* state;                // T [state_elems][3]
-    void* snap;                 // T [win_ring][M][3] parent at the start of window w, row w % win_ring
+    void* snap;                 // T [win_ring][M][3] parent at the start of window w, row w % win_ring (written
+                                // by the parent kernel that ends window w - 1, or by bd_set_positions)
     double* part_hist;          // [win_ring][part_stride] per-group replica sums, window w at w % win_ring
     double* tsf_hist;           // [max_windows][M] parent window means
     double* tsf_acc;            // [M] parent's running sum inside the current window
@@ -115,6 +116,7 @@ struct StepParams {
     // replica kernels: the launch's windows split into n_parts runs of
     // win_per_part windows (item_range); every (item, part) is a unit of work
     int32_t n_parts, win_per_part;
+    int32_t store_state, pad_store;   // this launch holds its slots' last step of the chunk
     void* conf_scratch;         // T [warps][kConfSlots L][3] window-end bonds of a warp's replicas (Eq. 5)
     double dt, s_min;
     int32_t S, flags, thr_mask, bell_mask;
@@ -144,7 +146,7 @@ __device__ __forceinline__ StepRange item_range(const StepParams& p, int part)
     r.t1 = (uint32_t)(e < end ? e : end);
     r.w = (int32_t)wf;
     r.s_in = (int32_t)(a - wf * p.S);
-    r.last = part + 1 == p.n_parts;
+    r.last = part + 1 == p.n_parts && p.store_state;
     return r;
 }
 

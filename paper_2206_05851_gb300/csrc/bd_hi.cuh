@@ -703,13 +703,10 @@ __device__ __forceinline__ void hi_parent_body(const StepParams& p, typename E::
     const int64_t t_end = p.t0 + p.n_steps;
 #pragma unroll 1
     for (int64_t t = p.t0; t < t_end; ++t) {
-        if (s_in == 0) {  // the conformation the replicas of window w start from
-            T* row = snap + ((w % p.win_ring) * M + ch.spr_off) * 3;
-            hi_store_bonds(sm, row, N);
-            // continue from it as the replicas do, so that replicas drawing
-            // the parent's noise repeat the parent exactly
-            hi_load_bonds(sm, row, N);
-        }
+        // the conformation the replicas of window w start from: continue from
+        // it as they do, so that replicas drawing the parent's noise repeat
+        // the parent exactly
+        if (s_in == 0) hi_load_bonds(sm, snap + ((w % p.win_ring) * M + ch.spr_off) * 3, N);
         floored += eng.step(sm, ch, k, kl, p, N, 0u, (uint32_t)c + p.chain_base, (uint32_t)t, harmonic, lj);
         if (eng.failed()) break;
         if (mine) {
@@ -744,16 +741,37 @@ __device__ __forceinline__ void hi_parent_body(const StepParams& p, typename E::
                 sums.next_window(rem);
             }
             ++w;
+            hi_store_bonds(sm, snap + ((w % p.win_ring) * M + ch.spr_off) * 3, N);
+            __syncthreads();          // read back by other threads (hi_load_bonds)
         }
     }
     eng.end(sm, p.dev_err);
     __syncthreads();
     hi_store_bonds(sm, state, N);
+    if (s_in == 0 && p.store_state) {      // the next chunk starts from positions rebuilt from the state
+        __syncthreads();
+        hi_load_bonds(sm, state, N);
+        hi_store_bonds(sm, snap + ((w % p.win_ring) * M + ch.spr_off) * 3, N);
+    }
     if (mine) {
         p.tsf_acc[m] = sums.tsf_sum();
         if (isf_bell) p.lam[CRIT_Q_ISF * M + m] += sums.hazard();
     }
     if (floored) atomicAdd(p.overext + c, (unsigned long long)floored);
+}
+
+// The snapshot of the window that starts at step t0, from the parents' state
+// (one CTA per parent; bd_set_positions), by way of the positions as the
+// kernels above take it.
+template <typename T> struct HISnapShared { T pos[3 * kHIMaxBeads], com[3]; };
+template <typename T>
+__global__ void __launch_bounds__(kHIThreads) hi_snap_kernel(const StepParams p)
+{
+    __shared__ HISnapShared<T> sm;
+    const int c = p.parent_items[p.parent_warps[blockIdx.x].first];
+    const ChainDev& ch = p.chains[c];
+    hi_load_bonds(sm, reinterpret_cast<const T*>(p.state) + ch.state_off * 3, ch.N);
+    hi_store_bonds(sm, reinterpret_cast<T*>(p.snap) + (((p.t0 / p.S) % p.win_ring) * p.M + ch.spr_off) * 3, ch.N);
 }
 
 template <typename T, bool FAST, int NTM>

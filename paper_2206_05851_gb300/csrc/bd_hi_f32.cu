@@ -28,6 +28,11 @@ const void* hi_parent_func_f32(bool small)
     return small ? (const void*)hi_parent_kernel<float, true, kHINTSmall>
                  : (const void*)hi_parent_kernel<float, true, kHINTMax>;
 }
+cudaError_t run_hi_snap_f32(int parents, const StepParams& p, cudaStream_t st)
+{
+    hi_snap_kernel<float><<<parents, kHIThreads, 0, st>>>(p);
+    return cudaGetLastError();
+}
 size_t hi_smem_f32(bool small)
 {
     if (small && BD_HI_TC) return sizeof(HITCShared);

@@ -19,6 +19,11 @@ const void* hi_parent_func_f64(bool small)
     return small ? (const void*)hi_parent_kernel<double, false, kHINTSmall>
                  : (const void*)hi_parent_kernel<double, false, kHINTMax>;
 }
+cudaError_t run_hi_snap_f64(int parents, const StepParams& p, cudaStream_t st)
+{
+    hi_snap_kernel<double><<<parents, kHIThreads, 0, st>>>(p);
+    return cudaGetLastError();
+}
 size_t hi_smem_f64(bool small)
 {
     return small ? sizeof(HIShared<double, kHINTSmall>) : sizeof(HIShared<double, kHINTMax>);

@@ -50,6 +50,8 @@ const void* hi_replica_func_f32(bool small);
 const void* hi_replica_func_f64(bool small);
 const void* hi_parent_func_f32(bool small);
 const void* hi_parent_func_f64(bool small);
+cudaError_t run_hi_snap_f32(int parents, const StepParams& p, cudaStream_t st);
+cudaError_t run_hi_snap_f64(int parents, const StepParams& p, cudaStream_t st);
 size_t hi_smem_f32(bool small);
 size_t hi_smem_f64(bool small);
 int hi_threads_f32(bool small);        // threads of a CTA of these kernels

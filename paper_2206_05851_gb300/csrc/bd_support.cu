@@ -31,10 +31,11 @@ __global__ void exp1_kernel(const ChainDev* chains, const int32_t* spring_chain,
     }
 }
 
-// Parent and every replica of spring m's chain <- r_{i+1} - r_i.
+// Parent and every replica of spring m's chain, and the parent's row of the
+// snapshot that the starting window's replicas copy, <- r_{i+1} - r_i.
 template <typename T>
 __global__ void set_bonds_kernel(const ChainDev* chains, const int32_t* spring_chain, int64_t M,
-                                 const double* pos, T* state)
+                                 const double* pos, T* state, T* snap_row)
 {
     const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
@@ -43,6 +44,7 @@ __global__ void set_bonds_kernel(const ChainDev* chains, const int32_t* spring_c
     const int nb = ch.N - 1;
     const double* r = pos + 3 * (ch.bead_off + i);
     const T q0 = (T)(r[3] - r[0]), q1 = (T)(r[4] - r[1]), q2 = (T)(r[5] - r[2]);
+    snap_row[3 * m] = q0; snap_row[3 * m + 1] = q1; snap_row[3 * m + 2] = q2;
     for (int s = 0; s <= ch.R; ++s) {
         T* d = state + 3 * (ch.state_off + (int64_t)s * nb + i);
         d[0] = q0; d[1] = q1; d[2] = q2;
@@ -354,11 +356,11 @@ cudaError_t run_exp1(const ChainDev* chains, const int32_t* spring_chain, int64_
 }
 
 cudaError_t run_set_bonds(bool f64, const ChainDev* chains, const int32_t* spring_chain, int64_t M,
-                          const double* pos, void* state, cudaStream_t st)
+                          const double* pos, void* state, void* snap_row, cudaStream_t st)
 {
     if (M == 0) return cudaSuccess;
-    if (f64) set_bonds_kernel<double><<<blocks_for(M), kThreads, 0, st>>>(chains, spring_chain, M, pos, (double*)state);
-    else set_bonds_kernel<float><<<blocks_for(M), kThreads, 0, st>>>(chains, spring_chain, M, pos, (float*)state);
+    if (f64) set_bonds_kernel<double><<<blocks_for(M), kThreads, 0, st>>>(chains, spring_chain, M, pos, (double*)state, (double*)snap_row);
+    else set_bonds_kernel<float><<<blocks_for(M), kThreads, 0, st>>>(chains, spring_chain, M, pos, (float*)state, (float*)snap_row);
     return cudaGetLastError();
 }
 

@@ -9,7 +9,8 @@
 //
 // Two kernels share one step routine:
 //   parent_kernel  advances every parent, writes its conformation at each
-//                  window start (the "halted parent" that replicas copy), and
+//                  window end (the "halted parent" that the next window's
+//                  replicas copy; bd_set_positions writes the first), and
 //                  samples it every step (ISF criteria, TSF sums);
 //   replica_kernel one CTA per (chain, replica group) evolves the replicas
 //                  window after window: spawn from the parent snapshot, S
@@ -44,8 +45,8 @@ namespace bdra {
 // Replicas, one warp work item (one replica per lane run). Lane run s of the
 // warp is replica rep_begin + stride s + 1; state of replica k lives at
 // state[(state_off + k (N-1)) * 3 ...]. Snapshots: snap[((w % win_ring) * M +
-// spr_off + i) * 3 + d], written by the parent kernel at every window start
-// of the current chunk. wsm: this warp's scratch of kWarpScratch values.
+// spr_off + i) * 3 + d], written by the parent kernel at the end of the
+// window before. wsm: this warp's scratch of kWarpScratch values.
 // ---------------------------------------------------------------------------
 constexpr int kWarpScratch = 512;   // >= slots per warp x springs = P (N-1) <= 32 L
 
@@ -345,8 +346,6 @@ parent_block_kernel(const StepParams p)
             T* brow = bonds + (b & 1) * (B * 3 * E);
 #pragma unroll 1
             for (int s = 0; s < nb_steps; ++s, nrow += 3 * E, brow += 3 * E) {
-                if (s_in == 0)   // the conformation the replicas of window w start from
-                    store_bonds<T, L>(qx, qy, qz, snap + ((w % p.win_ring) * M + spr_off) * 3, lc);
                 T dx[L], dy[L], dz[L];
                 row_load<T, L>(nrow, lane, dx);
                 row_load<T, L>(nrow + E, lane, dy);
@@ -355,7 +354,11 @@ parent_block_kernel(const StepParams p)
                 row_store<T, L>(brow, lane, qx);
                 row_store<T, L>(brow + E, lane, qy);
                 row_store<T, L>(brow + 2 * E, lane, qz);
-                if (++s_in == p.S) { s_in = 0; ++w; }
+                if (++s_in == p.S) {   // the conformation the replicas of the next window start from
+                    s_in = 0;
+                    ++w;
+                    store_bonds<T, L>(qx, qy, qz, snap + ((w % p.win_ring) * M + spr_off) * 3, lc);
+                }
             }
         }
         store_bonds<T, L>(qx, qy, qz, state, lc);
@@ -535,8 +538,6 @@ parent_kernel(const StepParams p)
     const int64_t t_end = p.t0 + p.n_steps;
 #pragma unroll 1
     for (int64_t t = p.t0; t < t_end; ++t) {
-        if (s_in == 0)   // the conformation the replicas of window w start from
-            store_bonds<T, L>(qx, qy, qz, snap + ((w % p.win_ring) * M + ch.spr_off) * 3, lc);
         if constexpr (LJ)
             floored += step_bonds_lj<T, L, FAST, true, 0>(qx, qy, qz, lc, k, kl, sw < P, sw < P ? lane - sw * G : 0, G,
                                             sw < P ? sw * G : lane, (uint32_t)t, p, my_tab);
@@ -584,6 +585,8 @@ parent_kernel(const StepParams p)
                 }
             }
             ++w;
+            // the conformation the replicas of the next window start from
+            store_bonds<T, L>(qx, qy, qz, snap + ((w % p.win_ring) * M + ch.spr_off) * 3, lc);
         }
     }
     store_bonds<T, L>(qx, qy, qz, state, lc);
