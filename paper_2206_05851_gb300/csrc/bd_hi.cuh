@@ -159,8 +159,8 @@ __device__ __forceinline__ void hi_tiles_init(HITiles<T, MAXT>& tl, int NT)
 }
 
 // The bead pairs of a chain of N beads into sm.pair (once per kernel).
-template <typename T, int NTM>
-__device__ __forceinline__ void hi_pairs_init(HIShared<T, NTM>& sm, int N)
+template <typename SM>
+__device__ __forceinline__ void hi_pairs_init(SM& sm, int N)
 {
     for (int k = threadIdx.x; k < N * (N + 1) / 2; k += blockDim.x) {
         int bi, bj;
@@ -176,10 +176,10 @@ __device__ __forceinline__ void hi_pairs_init(HIShared<T, NTM>& sm, int N)
 // Entry (p, q) of tile (I, J) = (p >> 2, q >> 2) is element
 // (4 (p & 3) + (q & 3)) kTiles + J NT - J (J + 1) / 2 + I of the tile copy:
 // a part of the row p plus a part of the column q.
-template <typename T, bool FAST, int NTM>
-__device__ __forceinline__ void hi_assemble(HIShared<T, NTM>& sm, int N, T a)
+template <typename T, bool FAST, typename SM>
+__device__ __forceinline__ void hi_assemble(SM& sm, int N, T a)
 {
-    constexpr int kT = HIShared<T, NTM>::kTiles;
+    constexpr int kT = SM::kTiles;
     const int pairs = N * (N + 1) / 2;
     const int NT = (3 * N + 3) / 4;
     T* tiles = &sm.st.tiles[0][0];
@@ -441,6 +441,30 @@ __device__ __forceinline__ void hi_store_bonds(const SM& sm, T* bonds, int N)
     for (int e = threadIdx.x; e < 3 * (N - 1); e += blockDim.x) bonds[e] = sm.pos[e + 3] - sm.pos[e];
 }
 
+// Positions to the centre-of-mass frame (every thread; after a barrier).
+template <typename T, typename SM>
+__device__ __forceinline__ void hi_centre(SM& sm, int N)
+{
+    const int tid = threadIdx.x;
+    if (tid < 32) {
+        T s[3] = {T(0), T(0), T(0)};
+        for (int b = tid; b < N; b += 32)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) s[c] += sm.pos[3 * b + c];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+        }
+        if (tid == 0)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sm.com[c] = s[c] / (T)N;
+    }
+    __syncthreads();
+    if (tid < 3 * N) sm.pos[tid] -= sm.com[tid % 3];
+    __syncthreads();
+}
+
 // One step t -> t + 1 of the CTA's slot. Returns the thread's floor count.
 template <typename T, bool FAST, int NTM, int MAXT>
 __device__ __forceinline__ int hi_step(HIShared<T, NTM>& sm, HITiles<T, MAXT>& tl, const ChainDev& ch,
@@ -459,7 +483,7 @@ __device__ __forceinline__ int hi_step(HIShared<T, NTM>& sm, HITiles<T, MAXT>& t
         sm.xi[3 * tid + 1] = z1;
         sm.xi[3 * tid + 2] = z2;
     }
-    hi_assemble<T, FAST, NTM>(sm, N, (T)ch.hi_a);
+    hi_assemble<T, FAST>(sm, N, (T)ch.hi_a);
     __syncthreads();
     hi_load_tiles<T, NTM, MAXT>(tl, sm, n);
     __syncthreads();                   // the partial products below overwrite the tile copy
@@ -522,23 +546,7 @@ __device__ __forceinline__ int hi_step(HIShared<T, NTM>& sm, HITiles<T, MAXT>& t
     __syncthreads();
     if (tid < n) sm.pos[tid] = nv;
     __syncthreads();
-    if (tid < 32) {
-        T s[3] = {T(0), T(0), T(0)};
-        for (int b = tid; b < N; b += 32)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) s[c] += sm.pos[3 * b + c];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
-        }
-        if (tid == 0)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) sm.com[c] = s[c] / (T)N;
-    }
-    __syncthreads();
-    if (tid < n) sm.pos[tid] -= sm.com[tid % 3];
-    __syncthreads();
+    hi_centre<T>(sm, N);
     return floored;
 }
 
@@ -604,6 +612,221 @@ template <typename T, bool FAST, int NTM> struct HITileEngine {
                                         uint32_t chain, uint32_t t, bool harmonic, bool lj)
     {
         return hi_step<T, FAST, NTM, kMaxT>(sm, tl, ch, k, kl, p, N, NT, key, chain, t, harmonic, lj);
+    }
+    __device__ __forceinline__ bool failed() const { return false; }
+    __device__ __forceinline__ void end(Shared&, int32_t*) {}
+};
+
+// ---------------------------------------------------------------------------
+// Float64. The tensor's tiles stay in shared memory (95 KB for up to 50
+// beads), so that a thread needs 128 registers instead of 255 and an SM holds
+// two CTAs. The float64 pipe issues one warp instruction every 16 cycles, so a
+// step is bound either by its 9100 tile updates (64 multiply-adds each, 150 us
+// an SM) or, in one CTA alone, by the 38 diagonal tiles, each a serial chain of
+// roots and divisions on one thread: 406 us a step, the same for one CTA an SM
+// in the tile-register form above. Two CTAs overlap the one's chain with the
+// other's updates; an update reads 48 values from shared memory for its 64
+// multiply-adds, a tenth of the time that those take. The diagonal tile takes
+// its roots and their reciprocals from one reciprocal square root, and W F and
+// L xi are row sums over the tiles (one thread a row) instead of per-tile
+// partials. The float32 form of up to 64 beads stays with the register tiles.
+// ---------------------------------------------------------------------------
+template <int NTM> struct HIShared64 {
+    static constexpr int kTiles = HIDims<NTM>::tiles;
+    static constexpr int kPanel = 18;  // row stride: 16-byte rows, two-way conflicts at most
+    alignas(16) double pos[4 * NTM];
+    alignas(16) double frc[4 * NTM];
+    alignas(16) double xi[4 * NTM];
+    alignas(16) double diag[16];
+    alignas(16) double dinv[4];
+    alignas(16) double panel[NTM][kPanel];
+    static constexpr int kBeads = NTM <= kHINTSmall ? kHISmallBeads : kHIMaxBeads;
+    uint16_t pair[kBeads * (kBeads + 1) / 2];
+    uint16_t tij[kTiles];                     // tile t as (I << 8) | J
+    struct alignas(16) { double tiles[16][kTiles]; } st;
+    double com[3];
+};
+
+__device__ __forceinline__ void hi_chol4_64(double (&A)[16], double (&inv)[4])
+{
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        double s = A[5 * j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) s = fma(-A[4 * j + k], A[4 * j + k], s);
+        const double il = rsqrt(s);
+        A[5 * j] = s * il;
+        inv[j] = il;
+#pragma unroll
+        for (int i = j + 1; i < 4; ++i) {
+            double v = A[4 * i + j];
+#pragma unroll
+            for (int k = 0; k < j; ++k) v = fma(-A[4 * i + k], A[4 * j + k], v);
+            A[4 * i + j] = v * il;
+        }
+    }
+}
+
+// hi_cholesky on the shared tiles.
+template <int NTM>
+__device__ __forceinline__ void hi_cholesky64(HIShared64<NTM>& sm, int NT)
+{
+    const int tid = threadIdx.x, total = NT * (NT + 1) / 2;
+    auto diagonal = [&](double (&A)[16], int t) {
+        double inv[4];
+        hi_chol4_64(A, inv);
+        hi_st16(sm.diag, A);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sm.dinv[e] = inv[e];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) sm.st.tiles[e][t] = A[e];
+    };
+    if (tid == 0) {
+        double A[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) A[e] = sm.st.tiles[e][0];
+        diagonal(A, 0);
+    }
+    __syncthreads();
+    int base = 0;                              // tile (K, K)
+#pragma unroll 1
+    for (int K = 0; K < NT; ++K) {
+        const int next = base + NT - K;        // tile (K + 1, K + 1)
+        if (tid < NT - 1 - K) {
+            const int t = base + 1 + tid;
+            double A[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) A[e] = sm.st.tiles[e][t];
+            hi_trsm4(A, sm.diag, sm.dinv);
+            hi_st16(sm.panel[K + 1 + tid], A);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) sm.st.tiles[e][t] = A[e];
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int t = next + tid; t < total; t += kHIThreads) {
+            const int I = sm.tij[t] >> 8, J = sm.tij[t] & 0xFF;
+            double A[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) A[e] = sm.st.tiles[e][t];
+#pragma unroll
+            for (int k2 = 0; k2 < 2; ++k2) {       // two columns of the panel at a time
+                double li[8], lj[8];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const double2 a = *reinterpret_cast<const double2*>(&sm.panel[I][4 * r + 2 * k2]);
+                    const double2 b = *reinterpret_cast<const double2*>(&sm.panel[J][4 * r + 2 * k2]);
+                    li[2 * r] = a.x; li[2 * r + 1] = a.y;
+                    lj[2 * r] = b.x; lj[2 * r + 1] = b.y;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        A[4 * i + j] = fma(-li[2 * i], lj[2 * j], A[4 * i + j]);
+                        A[4 * i + j] = fma(-li[2 * i + 1], lj[2 * j + 1], A[4 * i + j]);
+                    }
+            }
+            if (t == next) {
+                diagonal(A, t);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) sm.st.tiles[e][t] = A[e];
+            }
+        }
+        __syncthreads();
+        base = next;
+    }
+}
+
+// One step t -> t + 1 of the CTA's slot in float64 (hi_step on shared tiles).
+template <int NTM>
+__device__ __forceinline__ int hi_step64(HIShared64<NTM>& sm, const ChainDev& ch, const StepConst<double, false>& k,
+                                         const LJConst<double>& kl, const StepParams& p, int N, int NT,
+                                         uint32_t slot_key, uint32_t chain, uint32_t step, bool harmonic, bool lj)
+{
+    const int n = 3 * N;
+    const int tid = threadIdx.x;
+    const int floored = hi_forces<double, false>(sm, N, k, kl, harmonic, lj);
+    if (tid < N) {
+        double z0, z1, z2;
+        bead_noise<double, false>((uint32_t)tid, slot_key, step, chain, p, z0, z1, z2);
+        sm.xi[3 * tid] = z0;
+        sm.xi[3 * tid + 1] = z1;
+        sm.xi[3 * tid + 2] = z2;
+    }
+    hi_assemble<double, false>(sm, N, ch.hi_a);
+    __syncthreads();
+    // row sums over the tiles of row I = tid / 4: entries (c, j) of (I, J), J <= I,
+    // and, by symmetry, (j, c) of (J, I), J > I
+    const int I = tid >> 2, c = tid & 3;
+    double u = 0.0;
+    if (tid < n) {
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+        for (int J = 0; J < NT; ++J) {
+            const bool low = J <= I;
+            const double* e = &sm.st.tiles[low ? 4 * c : c][low ? hi_tile(I, J, NT) : hi_tile(J, I, NT)];
+            const int d = (low ? 1 : 4) * HIShared64<NTM>::kTiles;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[j] = fma(e[j * d], sm.frc[4 * J + j], s[j]);
+        }
+        u = (s[0] + s[1]) + (s[2] + s[3]);
+    }
+    __syncthreads();                   // W is read before the factor overwrites it
+    hi_cholesky64(sm, NT);
+    double nv = 0.0;
+    if (tid < n) {
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+        for (int J = 0; J < I; ++J) {
+            const int t = hi_tile(I, J, NT);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[j] = fma(sm.st.tiles[4 * c + j][t], sm.xi[4 * J + j], s[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (j <= c) s[j] = fma(sm.st.tiles[4 * c + j][hi_tile(I, I, NT)], sm.xi[4 * I + j], s[j]);
+        const double w = (s[0] + s[1]) + (s[2] + s[3]);
+        const int x = tid % 3, b3 = tid - x;
+        const double r = sm.pos[tid];
+        const double fl = x == 0 ? fma(k.axz, sm.pos[b3 + 2], fma(k.axx, r, r)) : (x == 1 ? fma(k.ayy, r, r) : fma(k.azz, r, r));
+        nv = fma(k.cn, w, fma(k.cd, u, fl));
+    }
+    __syncthreads();
+    if (tid < n) sm.pos[tid] = nv;
+    __syncthreads();
+    hi_centre<double>(sm, N);
+    return floored;
+}
+
+template <int NTM> struct HIEngine64 {
+    using Shared = HIShared64<NTM>;
+    int NT;
+    __device__ __forceinline__ void begin(Shared& sm, int N, int32_t)
+    {
+        NT = (3 * N + 3) / 4;
+        for (int e = threadIdx.x; e < 4 * NTM; e += blockDim.x) {
+            sm.pos[e] = 0.0; sm.frc[e] = 0.0; sm.xi[e] = 0.0;
+        }
+        hi_pairs_init(sm, N);
+        // rows and columns past 3N (of the last tile row) are the identity's;
+        // the tensor's entries are never written there and the factor leaves them
+        for (int t = threadIdx.x; t < NT * (NT + 1) / 2; t += blockDim.x) {
+            int I, J;
+            hi_uncol(t, NT, I, J);
+            sm.tij[t] = (uint16_t)((I << 8) | J);
+            if (I == NT - 1)
+#pragma unroll
+                for (int e = 0; e < 16; ++e) sm.st.tiles[e][t] = (I == J && e % 5 == 0) ? 1.0 : 0.0;
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ int step(Shared& sm, const ChainDev& ch, const StepConst<double, false>& k,
+                                        const LJConst<double>& kl, const StepParams& p, int N, uint32_t key,
+                                        uint32_t chain, uint32_t t, bool harmonic, bool lj)
+    {
+        return hi_step64<NTM>(sm, ch, k, kl, p, N, NT, key, chain, t, harmonic, lj);
     }
     __device__ __forceinline__ bool failed() const { return false; }
     __device__ __forceinline__ void end(Shared&, int32_t*) {}
@@ -774,20 +997,27 @@ __global__ void __launch_bounds__(kHIThreads) hi_snap_kernel(const StepParams p)
     hi_store_bonds(sm, reinterpret_cast<T*>(p.snap) + (((p.t0 / p.S) % p.win_ring) * p.M + ch.spr_off) * 3, ch.N);
 }
 
+// The slot engine of a kernel: shared tiles in float64, register tiles in
+// float32 (chains of 51 to 64 beads; shorter ones run on the tensor cores).
+template <typename T, bool FAST, int NTM> struct HIEngineOf { using type = HITileEngine<T, FAST, NTM>; };
+template <bool FAST, int NTM> struct HIEngineOf<double, FAST, NTM> { using type = HIEngine64<NTM>; };
+
 template <typename T, bool FAST, int NTM>
-__global__ void __launch_bounds__(kHIThreads, (sizeof(T) == 4 && NTM <= kHINTSmall) ? 3 : 1)
+__global__ void __launch_bounds__(kHIThreads, NTM > kHINTSmall ? 1 : sizeof(T) == 4 ? 3 : 2)
 hi_replica_kernel(const StepParams p)
 {
+    using E = typename HIEngineOf<T, FAST, NTM>::type;
     extern __shared__ __align__(16) unsigned char hi_smem_raw[];
-    hi_replica_body<T, FAST, HITileEngine<T, FAST, NTM>>(p, *reinterpret_cast<HIShared<T, NTM>*>(hi_smem_raw));
+    hi_replica_body<T, FAST, E>(p, *reinterpret_cast<typename E::Shared*>(hi_smem_raw));
 }
 
 template <typename T, bool FAST, int NTM>
-__global__ void __launch_bounds__(kHIThreads, (sizeof(T) == 4 && NTM <= kHINTSmall) ? 3 : 1)
+__global__ void __launch_bounds__(kHIThreads, NTM > kHINTSmall ? 1 : sizeof(T) == 4 ? 3 : 2)
 hi_parent_kernel(const StepParams p)
 {
+    using E = typename HIEngineOf<T, FAST, NTM>::type;
     extern __shared__ __align__(16) unsigned char hi_smem_raw[];
-    hi_parent_body<T, FAST, HITileEngine<T, FAST, NTM>>(p, *reinterpret_cast<HIShared<T, NTM>*>(hi_smem_raw));
+    hi_parent_body<T, FAST, E>(p, *reinterpret_cast<typename E::Shared*>(hi_smem_raw));
 }
 
 }  // namespace bdra

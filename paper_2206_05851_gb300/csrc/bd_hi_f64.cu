@@ -26,7 +26,7 @@ cudaError_t run_hi_snap_f64(int parents, const StepParams& p, cudaStream_t st)
 }
 size_t hi_smem_f64(bool small)
 {
-    return small ? sizeof(HIShared<double, kHINTSmall>) : sizeof(HIShared<double, kHINTMax>);
+    return small ? sizeof(HIShared64<kHINTSmall>) : sizeof(HIShared64<kHINTMax>);
 }
 
 int hi_threads_f64(bool)

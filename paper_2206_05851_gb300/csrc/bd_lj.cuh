@@ -17,7 +17,7 @@
 namespace bdra {
 
 template <typename T, bool FAST> struct Rsqrt {
-    static __device__ __forceinline__ T rsqrt(T x) { return T(1) / sqrt(x); }
+    static __device__ __forceinline__ T rsqrt(T x) { return ::rsqrt(x); }
     static __device__ __forceinline__ T rcp(T x) { return T(1) / x; }
 };
 template <> struct Rsqrt<float, true> {
