@@ -7,13 +7,13 @@
 // (t0 = 3 max(0, N - 42), a bead boundary) form the trailing block T, held in
 // tensor memory (TMEM): thread i of warps 0-3 owns row i of T, TMEM lane i.
 // The first t0 <= 24 rows (the head) belong to the lanes of warp 4. Per step:
-//   - bead forces and normals (as the CUDA-core kernel), and the pair
-//     coefficients of W (Eq. 3) once per bead pair into shared memory;
-//   - every thread builds its own row of W (Eqs. 2-3, bead by bead), takes
-//     the mobility-weighted force u = (W F)_row, keeps the head columns in
-//     registers and stores the T columns to its TMEM lane;
-//   - head: warp 4 factors the head block (one row a lane; each column's
-//     root broadcast by one shuffle, its entries through shared memory); the
+//   - bead forces and normals (as the CUDA-core kernel), and W's blocks (Eqs.
+//     2-3), one bead pair a thread, into a shared copy of T;
+//   - every thread takes its own row of the copy, the mobility-weighted force
+//     u = (W F)_row on the way, and stores it to its TMEM lane; the head
+//     columns follow through the same place into registers;
+//   - head: warp 4 factors the head block (one row a lane, four columns at a
+//     time, their entries through shared memory); the
 //     T rows solve their head columns against it (X L^T = W_T,head) and
 //     T <- T - X X^T on the tensor cores;
 //   - panels of 32 columns of T: warp p factors the diagonal block of
@@ -46,18 +46,31 @@ static_assert(kTCBlocksPerSM * kTCCols <= 512, "TMEM columns of the resident CTA
 constexpr uint32_t kTCPolls = 1u << 20;  // polls of a completion barrier before giving up
 static_assert(3 * (kTCMaxBeads - 42) <= 3 * kTCHeadBeads, "head of the largest chain");
 
+constexpr int kTCRows = 126;             // rows of the trailing block at most (42 beads)
+constexpr int kTCStride = 132;           // row strides of the tensor's shared copies: 16-byte rows whose
+constexpr int kTCHeadStride = 28;        // vector loads, one row a lane, meet every bank once
+
 struct HITCShared {
-    alignas(128) float op_hi[128 * 32];  // the panel's factor rows (tf32 high parts), MMA operand layout
-    alignas(128) float op_lo[128 * 32];  // their remainders
-    alignas(16) float4 pe[kTCMaxBeads * (kTCMaxBeads - 1) / 2];   // bead pairs bi > bj: (sqrt(c_d) d, c_i)
+    // W's trailing block while it is assembled, then its head columns (every
+    // row of the chain), then the MMA operands
+    union alignas(128) {
+        float w[kTCRows * kTCStride];
+        float wh[3 * kTCMaxBeads * kTCHeadStride];
+        struct {
+            alignas(128) float op_hi[128 * 32];  // the panel's factor rows (tf32 high parts), MMA operand layout
+            alignas(128) float op_lo[128 * 32];  // their remainders
+        };
+    };
     alignas(16) float lt[32][32];        // factor of the current diagonal block, transposed: lt[k][j] = L[j][k]
-    alignas(16) float col[2][32];        // column k of the block being factored (two in flight)
+    alignas(16) float col[2][4][32];     // four columns of the block being factored (two sets in flight)
     alignas(16) float dinv[32];          // reciprocals of its diagonal
     alignas(16) float pos[4 * kHINTSmall];   // bead positions [3N] (COM frame)
     alignas(16) float frc[4 * kHINTSmall];   // bead forces [3N]
     alignas(16) float xi[4 * kHINTSmall];    // bead normals [3N]
     float com[3];
-    uint16_t pr[kTCMaxBeads * (kTCMaxBeads - 1) / 2];   // pair p as (bi << 8) | bj, p = bi (bi - 1) / 2 + bj
+    // bead pairs bi >= bj as (bi << 8) | bj: those of the trailing block in row
+    // order, then those with a head bead
+    uint16_t pr[kTCMaxBeads * (kTCMaxBeads + 1) / 2];
     uint32_t taddr;                      // TMEM address of the CTA's columns
     alignas(8) uint64_t bar_next;        // MMAs of the next panel's columns done
     alignas(8) uint64_t bar_rest;        // every MMA issued so far done
@@ -101,91 +114,133 @@ struct TCState {
     }
 };
 
-// Pair coefficients of W (Eq. 3) for the bead pairs bi > bj of the chain:
-// W's 3 x 3 block of the pair is c_d d d^T + c_i I (d = r_bj - r_bi, c_d > 0
-// in both branches of Eq. 3), stored as e = sqrt(c_d) d and c_i, so that an
-// entry is e_x e_y + c_i [x = y] and the transposed entries are equal bitwise.
-__device__ __forceinline__ void tc_pairs(HITCShared& sm, int N, float a)
+// The 3 x 3 blocks of W (Eqs. 2-3) of the bead pairs q0 <= q < q1 of sm.pr
+// into a shared copy of rows of `stride` floats, both triangles: the block of
+// a pair is c_d d d^T + c_i I (d = r_bj - r_bi, c_d > 0 in both branches of
+// Eq. 3), taken as e e^T + c_i I with e = sqrt(c_d) d, so that transposed
+// entries are equal bitwise; the diagonal blocks are the identity. Row r of W
+// is row r - r0 of the copy, columns start at column c0 of W and end before c1
+// (head columns: only one of a block's two places may lie inside).
+//
+// A pair a thread and whole rows back: building its own row bead by bead took
+// each thread 30 instructions a bead (coefficient load, selects, three broadcast
+// loads), 26% of a step; the copy costs a thread six pairs of 18 stores and a
+// row of 32 vector loads. It lies where the MMA operands come later.
+__device__ __forceinline__ void tc_blocks(HITCShared& sm, float* dst, int stride, int r0, int c0, int c1, int q0, int q1,
+                                          float a)
 {
-    const int np = N * (N - 1) / 2;
-    for (int q = threadIdx.x; q < np; q += blockDim.x) {
+#pragma unroll 1
+    for (int q = q0 + (int)threadIdx.x; q < q1; q += kTCThreads) {
         const int bi = sm.pr[q] >> 8, bj = sm.pr[q] & 0xFF;
-        const float dx = sm.pos[3 * bj] - sm.pos[3 * bi];
-        const float dy = sm.pos[3 * bj + 1] - sm.pos[3 * bi + 1];
-        const float dz = sm.pos[3 * bj + 2] - sm.pos[3 * bi + 2];
-        float ci, cd;
-        rpy_coef<float, true>(dx, dy, dz, a, ci, cd);
-        const float sc = sqrt_approx(cd);
-        sm.pe[q] = make_float4(sc * dx, sc * dy, sc * dz, ci);
+        float e[3], ci;
+        if (bi == bj) {
+            e[0] = e[1] = e[2] = 0.0f;
+            ci = 1.0f;
+        } else {
+            const float dx = sm.pos[3 * bj] - sm.pos[3 * bi];
+            const float dy = sm.pos[3 * bj + 1] - sm.pos[3 * bi + 1];
+            const float dz = sm.pos[3 * bj + 2] - sm.pos[3 * bi + 2];
+            float cd;
+            rpy_coef<float, true>(dx, dy, dz, a, ci, cd);
+            const float sc = sqrt_approx(cd);
+            e[0] = sc * dx; e[1] = sc * dy; e[2] = sc * dz;
+        }
+        const bool lower = 3 * bj >= c0 && 3 * bj < c1, upper = 3 * bi >= c0 && 3 * bi < c1;
+        float* lo = dst + (3 * bi - r0) * stride + 3 * bj - c0;      // rows of bi, columns of bj
+        float* up = dst + (3 * bj - r0) * stride + 3 * bi - c0;
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) {
+                const float w = __fmaf_rn(e[x], e[y], x == y ? ci : 0.0f);
+                if (lower) lo[x * stride + y] = w;
+                if (upper) up[y * stride + x] = w;
+            }
     }
 }
 
-// The pair table (once per kernel).
-__device__ __forceinline__ void tc_pairs_init(HITCShared& sm, int N)
+// The pair table (once per kernel): pairs of trailing beads (bj >= hb), then
+// those with a head bead.
+__device__ __forceinline__ void tc_pairs_init(HITCShared& sm, int N, int hb)
 {
-    for (int q = threadIdx.x; q < N * (N - 1) / 2; q += blockDim.x) {
-        int bi = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)q)) * 0.5f);
-        while (bi * (bi - 1) / 2 > q) --bi;
-        while ((bi + 1) * bi / 2 <= q) ++bi;
-        sm.pr[q] = (uint16_t)((bi << 8) | (q - bi * (bi - 1) / 2));
+    const int m = N - hb, trailing = m * (m + 1) / 2;
+    for (int q = threadIdx.x; q < N * (N + 1) / 2; q += blockDim.x) {
+        int bi, bj;
+        if (q < trailing) {
+            hi_untri(q, bi, bj);
+            bi += hb; bj += hb;
+        } else {                   // bj < hb: bead bi = 0, 1, .. with min(bi + 1, hb) partners each
+            const int h = q - trailing, tri = hb * (hb + 1) / 2;
+            if (h < tri) {
+                hi_untri(h, bi, bj);
+            } else {
+                bi = hb + (h - tri) / hb;
+                bj = (h - tri) % hb;
+            }
+        }
+        sm.pr[q] = (uint16_t)((bi << 8) | bj);
     }
 }
 
-// Row r = 3 bi + x of W at the three columns of bead bj: W[r][3 bj + y],
-// zero unless `on`. Branch-free: the diagonal block reads any pair (the
-// first; N >= 2) and takes the identity by selects, and bj past the chain
-// is clamped for the read.
-__device__ __forceinline__ void tc_w3(const HITCShared& sm, int bi, int x, int bj, int N, bool on, float& w0,
-                                      float& w1, float& w2)
-{
-    const int bc = bj < N ? bj : N - 1;
-    const int hi = bi > bc ? bi : bc, lo = bi > bc ? bc : bi;
-    const bool same = hi == lo;
-    const float4 e = sm.pe[same ? 0 : hi * (hi - 1) / 2 + lo];
-    const float ex = same ? 0.0f : (x == 0 ? e.x : (x == 1 ? e.y : e.z));
-    const float ci = same ? 1.0f : e.w;
-    w0 = on ? __fmaf_rn(ex, e.x, x == 0 ? ci : 0.0f) : 0.0f;
-    w1 = on ? __fmaf_rn(ex, e.y, x == 1 ? ci : 0.0f) : 0.0f;
-    w2 = on ? __fmaf_rn(ex, e.z, x == 2 ? ci : 0.0f) : 0.0f;
-}
-
-// Lower Cholesky factor of a K x K block held one row a lane (A[j], j < K;
-// rows beyond the block are identity rows). Column k: lane k takes the
-// reciprocal square root of its diagonal and broadcasts it, the rows below
-// scale their entry, and every row subtracts the column's outer product from
-// its later entries, the column read from shared memory (two buffers). Each
-// lane also keeps its own diagonal entry in a register, updated with its own
-// column entries, so that the next column's root waits on one shuffle only.
-// Returns 1 / L[lane][lane].
+// Lower Cholesky factor of a K x K block (K a multiple of 4) held one row a
+// lane (A[j], j < K; rows beyond the block are identity rows), four columns at
+// a time. The columns are a serial chain and one warp works on it, so its
+// latency is all that counts: a column by itself is a reciprocal root on its
+// owner, a shuffle, and a pass of the column through shared memory before the
+// next root's entry is right (140 cycles). The 4 x 4 diagonal block's ten
+// entries are shuffled to every lane instead, each lane factors it by itself
+// (four roots, no exchange between them), solves its own four entries against
+// it, and the four columns pass through shared memory together for the update
+// of the later ones. Every entry takes the same operations in the same order
+// as column by column. Returns 1 / L[lane][lane].
 template <int K>
-__device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*col)[32])
+__device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*col)[4][32])
 {
-    float own_inv = 1.0f, dg = 0.0f;
+    float own_inv = 1.0f;
 #pragma unroll
-    for (int j = 0; j < K; ++j)
-        if (j == lane) dg = A[j];
+    for (int k = 0; k < K; k += 4) {
+        float d[4][4], il[4];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float il = __shfl_sync(0xffffffffu, Rsqrt<float, true>::rsqrt(dg), k);
-        if (lane == k) {
-            A[k] = __fmul_rn(dg, il);
-            own_inv = il;
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c <= r; ++c) d[r][c] = __shfl_sync(0xffffffffu, A[k + c], k + r);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            il[c] = Rsqrt<float, true>::rsqrt(d[c][c]);
+#pragma unroll
+            for (int r = c + 1; r < 4; ++r) d[r][c] = __fmul_rn(d[r][c], il[c]);
+#pragma unroll
+            for (int c2 = c + 1; c2 < 4; ++c2)
+#pragma unroll
+                for (int r = c2; r < 4; ++r) d[r][c2] = __fmaf_rn(-d[r][c], d[c2][c], d[r][c2]);
         }
-        const float lk = lane > k ? __fmul_rn(A[k], il) : 0.0f;
-        if (lane > k) {
-            A[k] = lk;
-            dg = __fmaf_rn(-lk, lk, dg);
+        // the lane's entries of the four columns: below its diagonal the solve,
+        // on it the root, above it what was there (never used)
+        float x[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float v = A[k + c];
+#pragma unroll
+            for (int c2 = 0; c2 < c; ++c2) v = __fmaf_rn(-x[c2], d[c][c2], v);
+            x[c] = lane >= k + c ? __fmul_rn(v, il[c]) : 0.0f;
+            if (lane == k + c) own_inv = il[c];
+            if (lane >= k + c) A[k + c] = x[c];
         }
-        if (k + 1 < K) {
-            col[k & 1][lane] = lk;
+        if (k + 4 < K) {
+            float (&buf)[4][32] = col[(k >> 2) & 1];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) buf[c][lane] = x[c];
             __syncwarp();
 #pragma unroll
-            for (int j4 = (k + 1) & ~3; j4 < K; j4 += 4) {
-                const float4 c = *reinterpret_cast<const float4*>(&col[k & 1][j4]);
-                if (j4 + 0 > k) A[j4 + 0] = __fmaf_rn(-lk, c.x, A[j4 + 0]);
-                if (j4 + 1 > k) A[j4 + 1] = __fmaf_rn(-lk, c.y, A[j4 + 1]);
-                if (j4 + 2 > k) A[j4 + 2] = __fmaf_rn(-lk, c.z, A[j4 + 2]);
-                if (j4 + 3 > k) A[j4 + 3] = __fmaf_rn(-lk, c.w, A[j4 + 3]);
+            for (int j4 = k + 4; j4 < K; j4 += 4) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float4 l = *reinterpret_cast<const float4*>(&buf[c][j4]);
+                    A[j4 + 0] = __fmaf_rn(-x[c], l.x, A[j4 + 0]);
+                    A[j4 + 1] = __fmaf_rn(-x[c], l.y, A[j4 + 1]);
+                    A[j4 + 2] = __fmaf_rn(-x[c], l.z, A[j4 + 2]);
+                    A[j4 + 3] = __fmaf_rn(-x[c], l.w, A[j4 + 3]);
+                }
             }
         }
     }
@@ -278,7 +333,8 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int t0 = ts.t0, m = ts.m, hb = ts.hb, P = ts.P;
     const int floored = hi_forces<float, true>(sm, N, k, kl, harmonic, lj);
-    tc_pairs(sm, N, (float)ch.hi_a);
+    const int trailing = (N - hb) * (N - hb + 1) / 2;       // pairs of trailing beads
+    tc_blocks(sm, sm.w, kTCStride, t0, t0, 3 * N, 0, trailing, (float)ch.hi_a);
     if (tid < N) {
         float z0, z1, z2;
         bead_noise<float, true>((uint32_t)tid, slot_key, step, chain, p, z0, z1, z2);
@@ -294,54 +350,55 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
     const bool head = warp == 4;
     const int row = head ? lane : t0 + tid;
     const bool valid = head ? lane < t0 : tid < m;
-    const int bi = valid ? row / 3 : 0, x = valid ? row - 3 * (row / 3) : 0;
     float A[32];
     float w = 0.0f;
-    float u0 = 0.0f, u1 = 0.0f, u2 = 0.0f;     // (W F)_row over the columns of each component
+    float u[3] = {0.0f, 0.0f, 0.0f};           // (W F)_row over the columns of each component, bead by bead
     if (!head) {
-#pragma unroll 1
-        for (int q = 0; q < 6; ++q) {         // TMEM columns [24 q, 24 q + 24): beads hb + 8 q ..
-            float V[24];
+        const float* src = sm.w + (valid ? tid : 0) * kTCStride;
 #pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                const int bj = hb + 8 * q + b;
-                float w0, w1, w2;
-                tc_w3(sm, bi, x, bj, N, valid && bj < N, w0, w1, w2);
-                const int fb = 3 * (bj < N ? bj : N - 1);
-                u0 = __fmaf_rn(w0, sm.frc[fb], u0);
-                u1 = __fmaf_rn(w1, sm.frc[fb + 1], u1);
-                u2 = __fmaf_rn(w2, sm.frc[fb + 2], u2);
-                V[3 * b] = w0; V[3 * b + 1] = w1; V[3 * b + 2] = w2;
+        for (int g = 0; g < 16; ++g) {         // TMEM columns [8 g, 8 g + 8)
+            float V[8];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float4 v = *reinterpret_cast<const float4*>(src + 8 * g + 4 * q);
+                V[4 * q] = v.x; V[4 * q + 1] = v.y; V[4 * q + 2] = v.z; V[4 * q + 3] = v.w;
             }
-            tc::tmem_st8(ts.taddr + 24 * q, V);
-            if (q < 5) {
-                tc::tmem_st8(ts.taddr + 24 * q + 8, V + 8);
-                tc::tmem_st8(ts.taddr + 24 * q + 16, V + 16);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int c = 8 * g + e;
+                if (!(valid && c < m)) V[e] = 0.0f;      // past the block the copy holds anything
+                if (c < kTCRows) u[c % 3] = __fmaf_rn(V[e], sm.frc[t0 + c], u[c % 3]);
             }
-        }
-    } else if (valid) {
-#pragma unroll 4
-        for (int bj = hb; bj < N; ++bj) {
-            float w0, w1, w2;
-            tc_w3(sm, bi, x, bj, N, true, w0, w1, w2);
-            u0 = __fmaf_rn(w0, sm.frc[3 * bj], u0);
-            u1 = __fmaf_rn(w1, sm.frc[3 * bj + 1], u1);
-            u2 = __fmaf_rn(w2, sm.frc[3 * bj + 2], u2);
+            tc::tmem_st8(ts.taddr + 8 * g, V);
         }
     }
 #pragma unroll
-    for (int b = 0; b < kTCHeadBeads; ++b) {
-        float w0, w1, w2;
-        tc_w3(sm, bi, x, b, N, valid && b < hb, w0, w1, w2);
-        const int fb = 3 * (b < N ? b : N - 1);
-        u0 = __fmaf_rn(w0, sm.frc[fb], u0);
-        u1 = __fmaf_rn(w1, sm.frc[fb + 1], u1);
-        u2 = __fmaf_rn(w2, sm.frc[fb + 2], u2);
-        A[3 * b] = w0; A[3 * b + 1] = w1; A[3 * b + 2] = w2;
-    }
-    const float u = __fadd_rn(__fadd_rn(u0, u1), u2);
+    for (int j = 0; j < 32; ++j) A[j] = 0.0f;
+    if (t0 > 0) {                              // (t0 is the CTA's)
+        __syncthreads();                       // the trailing block is read: its place takes the head columns
+        tc_blocks(sm, sm.wh, kTCHeadStride, 0, 0, t0, trailing, N * (N + 1) / 2, (float)ch.hi_a);
+        __syncthreads();
+        if (head && valid) {
+#pragma unroll 3
+            for (int c = t0; c < 3 * N; c += 3) {          // the row's trailing columns, by symmetry
+                u[0] = __fmaf_rn(sm.wh[c * kTCHeadStride + lane], sm.frc[c], u[0]);
+                u[1] = __fmaf_rn(sm.wh[(c + 1) * kTCHeadStride + lane], sm.frc[c + 1], u[1]);
+                u[2] = __fmaf_rn(sm.wh[(c + 2) * kTCHeadStride + lane], sm.frc[c + 2], u[2]);
+            }
+        }
+        const float* src = sm.wh + (valid ? row : 0) * kTCHeadStride;
 #pragma unroll
-    for (int j = 3 * kTCHeadBeads; j < 32; ++j) A[j] = 0.0f;
+        for (int q = 0; q < 6; ++q) {
+            const float4 v = *reinterpret_cast<const float4*>(src + 4 * q);
+            A[4 * q] = v.x; A[4 * q + 1] = v.y; A[4 * q + 2] = v.z; A[4 * q + 3] = v.w;
+        }
+#pragma unroll
+        for (int c = 0; c < 3 * kTCHeadBeads; ++c) {
+            if (!(valid && c < t0)) A[c] = 0.0f;
+            u[c % 3] = __fmaf_rn(A[c], sm.frc[c], u[c % 3]);
+        }
+    }
+    const float uf = __fadd_rn(__fadd_rn(u[0], u[1]), u[2]);
     if (head && !valid) {        // identity rows below the head block
 #pragma unroll
         for (int j = 0; j < 32; ++j) A[j] = j == lane ? 1.0f : 0.0f;
@@ -430,7 +487,7 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
         const float r = sm.pos[row];
         const float fl = xx == 0 ? fmaf(k.axz, sm.pos[b3 + 2], fmaf(k.axx, r, r))
                                  : (xx == 1 ? fmaf(k.ayy, r, r) : fmaf(k.azz, r, r));
-        nv = fmaf(k.cn, w, fmaf(k.cd, u, fl));
+        nv = fmaf(k.cn, w, fmaf(k.cd, uf, fl));
     }
     __syncthreads();
     if (valid) sm.pos[row] = nv;
@@ -464,7 +521,7 @@ __device__ __forceinline__ void hi_tc_begin(HITCShared& sm, TCState& ts, int N)
         tc::mbar_init(&sm.bar_rest, 1);
     }
     for (int e = threadIdx.x; e < 128 * 32; e += blockDim.x) sm.op_hi[e] = sm.op_lo[e] = 0.0f;
-    tc_pairs_init(sm, N);
+    tc_pairs_init(sm, N, N > 42 ? N - 42 : 0);
     if (warp == 0) {
         tc::tmem_alloc(&sm.taddr, kTCCols);
         tc::tmem_relinquish();
