@@ -390,11 +390,16 @@ __device__ __forceinline__ int hi_forces(SM& sm, int N, const StepConst<T, FAST>
         }
         if (lj) {
             const T x0 = sm.pos[3 * b], y0 = sm.pos[3 * b + 1], z0 = sm.pos[3 * b + 2];
-#pragma unroll 1
+            // (in float32 the bead itself and its neighbours are evaluated and
+            // dropped, so that four partners are in flight: 13 rounds of a load, a
+            // reciprocal and its products were 7600 cycles of a lone CTA's step)
+#pragma unroll (sizeof(T) == 4 ? 4 : 1)
             for (int j = q; j < N; j += 4) {
-                if (j == b || j == b - 1 || j == b + 1) continue;
+                const bool skip = j == b || j == b - 1 || j == b + 1;
+                if (sizeof(T) == 8 && skip) continue;
                 const T dx = sm.pos[3 * j] - x0, dy = sm.pos[3 * j + 1] - y0, dz = sm.pos[3 * j + 2] - z0;
-                const T c = lj_coef<T, FAST>(dx, dy, dz, kl);
+                const T cv = lj_coef<T, FAST>(dx, dy, dz, kl);
+                const T c = skip ? T(0) : cv;
                 f[0] = fma(c, dx, f[0]); f[1] = fma(c, dy, f[1]); f[2] = fma(c, dz, f[2]);
             }
         }

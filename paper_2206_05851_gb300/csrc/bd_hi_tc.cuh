@@ -197,6 +197,18 @@ template <int K>
 __device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*col)[4][32])
 {
     float own_inv = 1.0f;
+    float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    // rows j4 .. j4 + 3 of the update by the four columns in buf
+    auto update = [&](const float (&buf)[4][32], int j4) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float4 l = *reinterpret_cast<const float4*>(&buf[c][j4]);
+            A[j4 + 0] = __fmaf_rn(-x[c], l.x, A[j4 + 0]);
+            A[j4 + 1] = __fmaf_rn(-x[c], l.y, A[j4 + 1]);
+            A[j4 + 2] = __fmaf_rn(-x[c], l.z, A[j4 + 2]);
+            A[j4 + 3] = __fmaf_rn(-x[c], l.w, A[j4 + 3]);
+        }
+    };
 #pragma unroll
     for (int k = 0; k < K; k += 4) {
         float d[4][4], il[4];
@@ -204,6 +216,11 @@ __device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*
         for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int c = 0; c <= r; ++c) d[r][c] = __shfl_sync(0xffffffffu, A[k + c], k + r);
+        // the rest of the previous four columns' update fills the chain's waits
+        if (k > 0) {
+#pragma unroll
+            for (int j4 = k + 4; j4 < K; j4 += 4) update(col[((k >> 2) + 1) & 1], j4);
+        }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             il[c] = Rsqrt<float, true>::rsqrt(d[c][c]);
@@ -216,7 +233,6 @@ __device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*
         }
         // the lane's entries of the four columns: below its diagonal the solve,
         // on it the root, above it what was there (never used)
-        float x[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             float v = A[k + c];
@@ -231,38 +247,38 @@ __device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*
 #pragma unroll
             for (int c = 0; c < 4; ++c) buf[c][lane] = x[c];
             __syncwarp();
-#pragma unroll
-            for (int j4 = k + 4; j4 < K; j4 += 4) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float4 l = *reinterpret_cast<const float4*>(&buf[c][j4]);
-                    A[j4 + 0] = __fmaf_rn(-x[c], l.x, A[j4 + 0]);
-                    A[j4 + 1] = __fmaf_rn(-x[c], l.y, A[j4 + 1]);
-                    A[j4 + 2] = __fmaf_rn(-x[c], l.z, A[j4 + 2]);
-                    A[j4 + 3] = __fmaf_rn(-x[c], l.w, A[j4 + 3]);
-                }
-            }
+            update(buf, k + 4);                // the next four columns first
         }
     }
     return own_inv;
 }
 
-// A <- A L^{-T} (forward substitution over K columns) with the factor in
-// sm.lt / sm.dinv; columns whose factor rows are identity rows pass through.
+// A <- A L^{-T} (forward substitution over K columns, four at a time) with the
+// factor in sm.lt / sm.dinv; columns whose factor rows are identity rows pass
+// through.
 template <int K>
 __device__ __forceinline__ void tc_row_solve(float (&A)[32], const HITCShared& sm)
 {
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        A[k] = __fmul_rn(A[k], sm.dinv[k]);
+    for (int k = 0; k < K; k += 4) {
+        const float4 iv = *reinterpret_cast<const float4*>(&sm.dinv[k]);
+        const float4 l0 = *reinterpret_cast<const float4*>(&sm.lt[k][k]);
+        const float4 l1 = *reinterpret_cast<const float4*>(&sm.lt[k + 1][k]);
+        const float4 l2 = *reinterpret_cast<const float4*>(&sm.lt[k + 2][k]);
+        A[k] = __fmul_rn(A[k], iv.x);
+        A[k + 1] = __fmul_rn(__fmaf_rn(-A[k], l0.y, A[k + 1]), iv.y);
+        A[k + 2] = __fmul_rn(__fmaf_rn(-A[k + 1], l1.z, __fmaf_rn(-A[k], l0.z, A[k + 2])), iv.z);
+        A[k + 3] = __fmul_rn(__fmaf_rn(-A[k + 2], l2.w, __fmaf_rn(-A[k + 1], l1.w, __fmaf_rn(-A[k], l0.w, A[k + 3]))), iv.w);
 #pragma unroll
-        for (int j4 = (k + 1) & ~3; j4 < K; j4 += 4) {
-            const float4 l = *reinterpret_cast<const float4*>(&sm.lt[k][j4]);
-            if (j4 + 0 > k) A[j4 + 0] = __fmaf_rn(-A[k], l.x, A[j4 + 0]);
-            if (j4 + 1 > k && j4 + 1 < K) A[j4 + 1] = __fmaf_rn(-A[k], l.y, A[j4 + 1]);
-            if (j4 + 2 > k && j4 + 2 < K) A[j4 + 2] = __fmaf_rn(-A[k], l.z, A[j4 + 2]);
-            if (j4 + 3 > k && j4 + 3 < K) A[j4 + 3] = __fmaf_rn(-A[k], l.w, A[j4 + 3]);
-        }
+        for (int j4 = k + 4; j4 < K; j4 += 4)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float4 l = *reinterpret_cast<const float4*>(&sm.lt[k + c][j4]);
+                A[j4 + 0] = __fmaf_rn(-A[k + c], l.x, A[j4 + 0]);
+                A[j4 + 1] = __fmaf_rn(-A[k + c], l.y, A[j4 + 1]);
+                A[j4 + 2] = __fmaf_rn(-A[k + c], l.z, A[j4 + 2]);
+                A[j4 + 3] = __fmaf_rn(-A[k + c], l.w, A[j4 + 3]);
+            }
     }
 }
 
@@ -333,15 +349,17 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int t0 = ts.t0, m = ts.m, hb = ts.hb, P = ts.P;
     const int floored = hi_forces<float, true>(sm, N, k, kl, harmonic, lj);
+    // the normals on the last threads: the force pass's second round (beads past
+    // the 40th) keeps the first warps
+    if (const int b = tid - (kTCThreads - N); b >= 0) {
+        float z0, z1, z2;
+        bead_noise<float, true>((uint32_t)b, slot_key, step, chain, p, z0, z1, z2);
+        sm.xi[3 * b] = z0;
+        sm.xi[3 * b + 1] = z1;
+        sm.xi[3 * b + 2] = z2;
+    }
     const int trailing = (N - hb) * (N - hb + 1) / 2;       // pairs of trailing beads
     tc_blocks(sm, sm.w, kTCStride, t0, t0, 3 * N, 0, trailing, (float)ch.hi_a);
-    if (tid < N) {
-        float z0, z1, z2;
-        bead_noise<float, true>((uint32_t)tid, slot_key, step, chain, p, z0, z1, z2);
-        sm.xi[3 * tid] = z0;
-        sm.xi[3 * tid + 1] = z1;
-        sm.xi[3 * tid + 2] = z2;
-    }
     __syncthreads();
 
     // rows of W: T rows (warps 0-3) into TMEM, then their head columns into
@@ -379,7 +397,7 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
         tc_blocks(sm, sm.wh, kTCHeadStride, 0, 0, t0, trailing, N * (N + 1) / 2, (float)ch.hi_a);
         __syncthreads();
         if (head && valid) {
-#pragma unroll 3
+#pragma unroll 7
             for (int c = t0; c < 3 * N; c += 3) {          // the row's trailing columns, by symmetry
                 u[0] = __fmaf_rn(sm.wh[c * kTCHeadStride + lane], sm.frc[c], u[0]);
                 u[1] = __fmaf_rn(sm.wh[(c + 1) * kTCHeadStride + lane], sm.frc[c + 1], u[1]);
@@ -413,22 +431,21 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
 #pragma unroll
             for (int j = 0; j < 3 * kTCHeadBeads; ++j) sm.lt[j][lane] = A[j];
             sm.dinv[lane] = il;
-            if (valid)
-#pragma unroll
-                for (int j = 0; j < 3 * kTCHeadBeads; ++j)
-                    if (j <= lane) w = __fmaf_rn(A[j], sm.xi[j], w);
         }
         __syncthreads();
         if (!head) {
             tc_row_solve<3 * kTCHeadBeads>(A, sm);
-#pragma unroll
-            for (int j = 0; j < 3 * kTCHeadBeads; ++j) w = __fmaf_rn(A[j], sm.xi[j], w);
             tc_put_operand<2 * kTCHeadBeads * 3 / 8>(sm, tid, A, !valid);
         }
         tc::fence_async_smem();
         __syncthreads();
         if (tid == 0) tc_issue_two(sm, ts.taddr, 0, m, (t0 + 7) >> 3, ts.stall);
         ts.pend_next = ts.pend_rest = true;
+        // w = L xi, here and in the panels behind the barrier that others wait at
+        // (rows past T are zero rows in the head columns)
+#pragma unroll
+        for (int j = 0; j < 3 * kTCHeadBeads; ++j)
+            if (!head || (valid && j <= lane)) w = __fmaf_rn(A[j], sm.xi[j], w);
     }
 
     // panels of T
@@ -450,20 +467,11 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
 #pragma unroll
                 for (int j = 0; j < 32; ++j) sm.lt[j][lane] = A[j];
                 sm.dinv[lane] = il;
-                if (valid)
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (j <= lane) w = __fmaf_rn(A[j], sm.xi[t0 + c0 + j], w);
             }
         }
         ts.wait_rest(sm);          // the previous update no longer reads the operand
         tc_sync();
-        if (!head && warp > pn) {
-            tc_row_solve<32>(A, sm);
-            if (valid)
-#pragma unroll
-                for (int j = 0; j < 32; ++j) w = __fmaf_rn(A[j], sm.xi[t0 + c0 + j], w);
-        }
+        if (!head && warp > pn) tc_row_solve<32>(A, sm);
         if (pn + 1 < P) {
             if (!head && warp > pn) tc_put_operand<8>(sm, tid, A, !valid);
             tc::fence_async_smem();
@@ -473,6 +481,10 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
         } else {
             __syncthreads();       // every read of sm.lt done before the next step writes it
         }
+        if (!head && warp >= pn && valid)
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (warp > pn || j <= lane) w = __fmaf_rn(A[j], sm.xi[t0 + c0 + j], w);
     }
     ts.wait_next(sm);
     ts.wait_rest(sm);
