@@ -50,6 +50,8 @@ constexpr int kTCRows = 126;             // rows of the trailing block at most (
 constexpr int kTCStride = 132;           // row strides of the tensor's shared copies: 16-byte rows whose
 constexpr int kTCHeadStride = 28;        // vector loads, one row a lane, meet every bank once
 
+constexpr int kTCNB = 4;                 // columns the diagonal factor takes at a time (8: spills, 8% slower)
+
 struct HITCShared {
     // W's trailing block while it is assembled, then its head columns (every
     // row of the chain), then the MMA operands
@@ -62,7 +64,7 @@ struct HITCShared {
         };
     };
     alignas(16) float lt[32][32];        // factor of the current diagonal block, transposed: lt[k][j] = L[j][k]
-    alignas(16) float col[2][4][32];     // four columns of the block being factored (two sets in flight)
+    alignas(16) float col[2][kTCNB][32]; // columns of the block being factored (two sets in flight)
     alignas(16) float dinv[32];          // reciprocals of its diagonal
     alignas(16) float pos[4 * kHINTSmall];   // bead positions [3N] (COM frame)
     alignas(16) float frc[4 * kHINTSmall];   // bead forces [3N]
@@ -73,7 +75,7 @@ struct HITCShared {
     uint16_t pr[kTCMaxBeads * (kTCMaxBeads + 1) / 2];
     uint32_t taddr;                      // TMEM address of the CTA's columns
     alignas(8) uint64_t bar_next;        // MMAs of the next panel's columns done
-    alignas(8) uint64_t bar_rest;        // every MMA issued so far done
+    alignas(8) uint64_t bar_rest;        // MMAs of the columns after them done
 };
 
 // Per-thread bookkeeping of the CTA's tensor-memory state. Only thread 0
@@ -182,26 +184,28 @@ __device__ __forceinline__ void tc_pairs_init(HITCShared& sm, int N, int hb)
     }
 }
 
-// Lower Cholesky factor of a K x K block (K a multiple of 4) held one row a
-// lane (A[j], j < K; rows beyond the block are identity rows), four columns at
-// a time. The columns are a serial chain and one warp works on it, so its
-// latency is all that counts: a column by itself is a reciprocal root on its
-// owner, a shuffle, and a pass of the column through shared memory before the
-// next root's entry is right (140 cycles). The 4 x 4 diagonal block's ten
-// entries are shuffled to every lane instead, each lane factors it by itself
-// (four roots, no exchange between them), solves its own four entries against
-// it, and the four columns pass through shared memory together for the update
-// of the later ones. Every entry takes the same operations in the same order
-// as column by column. Returns 1 / L[lane][lane].
+// Lower Cholesky factor of a K x K block held one row a lane (A[j], j < K;
+// rows beyond the block are identity rows), NB columns at a time (K a multiple
+// of NB, NB of 4). The columns are a serial chain and one warp works on it, so
+// its latency is all that counts: a column by itself is a reciprocal root on
+// its owner, a shuffle, and a pass of the column through shared memory before
+// the next root's entry is right (140 cycles). The NB x NB diagonal block's
+// lower entries are shuffled to every lane instead, each lane factors it by
+// itself (NB roots, no exchange between them), solves its own NB entries
+// against it, and the columns pass through shared memory together for the
+// update of the later ones, the next NB first: the rest of it fills the next
+// block's waits. Every entry takes the same operations in the same order as
+// column by column. Returns 1 / L[lane][lane].
 template <int K>
-__device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*col)[4][32])
+__device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*col)[kTCNB][32])
 {
+    constexpr int NB = kTCNB;
     float own_inv = 1.0f;
-    float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    // rows j4 .. j4 + 3 of the update by the four columns in buf
-    auto update = [&](const float (&buf)[4][32], int j4) {
+    float x[NB];
+    // columns j4 .. j4 + 3 of the update by the NB columns in buf
+    auto update = [&](const float (&buf)[NB][32], int j4) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < NB; ++c) {
             const float4 l = *reinterpret_cast<const float4*>(&buf[c][j4]);
             A[j4 + 0] = __fmaf_rn(-x[c], l.x, A[j4 + 0]);
             A[j4 + 1] = __fmaf_rn(-x[c], l.y, A[j4 + 1]);
@@ -210,31 +214,30 @@ __device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*
         }
     };
 #pragma unroll
-    for (int k = 0; k < K; k += 4) {
-        float d[4][4], il[4];
+    for (int k = 0; k < K; k += NB) {
+        float d[NB][NB], il[NB];
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < NB; ++r)
 #pragma unroll
             for (int c = 0; c <= r; ++c) d[r][c] = __shfl_sync(0xffffffffu, A[k + c], k + r);
-        // the rest of the previous four columns' update fills the chain's waits
         if (k > 0) {
 #pragma unroll
-            for (int j4 = k + 4; j4 < K; j4 += 4) update(col[((k >> 2) + 1) & 1], j4);
+            for (int j4 = k + NB; j4 < K; j4 += 4) update(col[((k / NB) + 1) & 1], j4);
         }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < NB; ++c) {
             il[c] = Rsqrt<float, true>::rsqrt(d[c][c]);
 #pragma unroll
-            for (int r = c + 1; r < 4; ++r) d[r][c] = __fmul_rn(d[r][c], il[c]);
+            for (int r = c + 1; r < NB; ++r) d[r][c] = __fmul_rn(d[r][c], il[c]);
 #pragma unroll
-            for (int c2 = c + 1; c2 < 4; ++c2)
+            for (int c2 = c + 1; c2 < NB; ++c2)
 #pragma unroll
-                for (int r = c2; r < 4; ++r) d[r][c2] = __fmaf_rn(-d[r][c], d[c2][c], d[r][c2]);
+                for (int r = c2; r < NB; ++r) d[r][c2] = __fmaf_rn(-d[r][c], d[c2][c], d[r][c2]);
         }
-        // the lane's entries of the four columns: below its diagonal the solve,
-        // on it the root, above it what was there (never used)
+        // the lane's entries of the columns: below its diagonal the solve, on it
+        // the root, above it what was there (never used)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < NB; ++c) {
             float v = A[k + c];
 #pragma unroll
             for (int c2 = 0; c2 < c; ++c2) v = __fmaf_rn(-x[c2], d[c][c2], v);
@@ -242,12 +245,13 @@ __device__ __forceinline__ float tc_warp_chol(float (&A)[32], int lane, float (*
             if (lane == k + c) own_inv = il[c];
             if (lane >= k + c) A[k + c] = x[c];
         }
-        if (k + 4 < K) {
-            float (&buf)[4][32] = col[(k >> 2) & 1];
+        if (k + NB < K) {
+            float (&buf)[NB][32] = col[(k / NB) & 1];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) buf[c][lane] = x[c];
+            for (int c = 0; c < NB; ++c) buf[c][lane] = x[c];
             __syncwarp();
-            update(buf, k + 4);                // the next four columns first
+#pragma unroll
+            for (int j4 = k + NB; j4 < k + 2 * NB; j4 += 4) update(buf, j4);
         }
     }
     return own_inv;
@@ -300,36 +304,43 @@ __device__ __forceinline__ void tc_put_operand(HITCShared& sm, int row, const fl
     }
 }
 
-// T[:, c0 .. c0 + N) -= X X[c0 .. c0 + N)^T over ks K steps of 8, X the
-// operand rows (three tf32 products per step).
+// T[:, c0 .. c0 + N) -= X X[c0 .. c0 + N)^T over ks K steps of 8, X
+// the operand rows (three tf32 products per step). The descriptors of all
+// steps are the first one's plus 256 bytes a step (address field in 16 bytes).
 __device__ __forceinline__ void tc_issue_update(HITCShared& sm, uint32_t tbase, int c0, int N, int ks)
 {
     const uint32_t id = tc::idesc_tf32(128, N, true);
     const uint32_t hi = tc::smem_u32(sm.op_hi), lo = tc::smem_u32(sm.op_lo);
-    const uint32_t boff = (uint32_t)(c0 >> 3) * 1024u;
-#pragma unroll 1
+    const uint32_t boff = (uint32_t)(c0 >> 3) * 1024u, d = tbase + (uint32_t)c0;
+    const uint64_t ah = tc::smem_desc(hi, 128, 1024), al = tc::smem_desc(lo, 128, 1024);
+    const uint64_t bh = tc::smem_desc(hi + boff, 128, 1024), bl = tc::smem_desc(lo + boff, 128, 1024);
+#pragma unroll 1                             // (unrolled: 1.5% slower)
     for (int s = 0; s < ks; ++s) {
-        const uint32_t ko = 256u * (uint32_t)s;
-        const uint64_t ah = tc::smem_desc(hi + ko, 128, 1024), al = tc::smem_desc(lo + ko, 128, 1024);
-        const uint64_t bh = tc::smem_desc(hi + boff + ko, 128, 1024), bl = tc::smem_desc(lo + boff + ko, 128, 1024);
-        tc::mma_tf32(tbase + (uint32_t)c0, ah, bh, id, true);
-        tc::mma_tf32(tbase + (uint32_t)c0, ah, bl, id, true);
-        tc::mma_tf32(tbase + (uint32_t)c0, al, bh, id, true);
+        tc::mma_tf32(d, ah + 16 * s, bh + 16 * s, id, true);
+        tc::mma_tf32(d, ah + 16 * s, bl + 16 * s, id, true);
+        tc::mma_tf32(d, al + 16 * s, bh + 16 * s, id, true);
     }
 }
 
-// The two-part update after a panel (or the head): next panel's columns
-// [c1, c1 + 32), then the rest up to the padded width of T. Thread 0 only.
-// With `stall` (a failure test) nothing is issued, so the waits give up.
+// The two-part update after a panel (or the head): thread 0 issues the next
+// panel's columns [c1, c1 + 32) and its completion (bar_next), thread
+// kTCSecond the rest up to the padded width of T (bar_rest): one thread
+// needs 2000 cycles to issue all 24 MMAs, longer than they run (800). With `stall` (a
+// failure test) nothing is issued, so the waits give up.
+constexpr int kTCSecond = 128;
 __device__ __forceinline__ void tc_issue_two(HITCShared& sm, uint32_t tbase, int c1, int m, int ks, bool stall)
 {
     if (stall) return;
-    tc::fence_after_sync();
-    tc_issue_update(sm, tbase, c1, 32, ks);
-    tc::mma_commit(&sm.bar_next);
-    const int width = (m + 15) & ~15;
-    if (c1 + 32 < width) tc_issue_update(sm, tbase, c1 + 32, width - c1 - 32, ks);
-    tc::mma_commit(&sm.bar_rest);
+    if (threadIdx.x == 0) {
+        tc::fence_after_sync();
+        tc_issue_update(sm, tbase, c1, 32, ks);
+        tc::mma_commit(&sm.bar_next);
+    } else if (threadIdx.x == kTCSecond) {
+        tc::fence_after_sync();
+        const int width = (m + 15) & ~15;
+        if (c1 + 32 < width) tc_issue_update(sm, tbase, c1 + 32, width - c1 - 32, ks);
+        tc::mma_commit(&sm.bar_rest);
+    }
 }
 
 __device__ __forceinline__ void tc_sync()
@@ -439,7 +450,7 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
         }
         tc::fence_async_smem();
         __syncthreads();
-        if (tid == 0) tc_issue_two(sm, ts.taddr, 0, m, (t0 + 7) >> 3, ts.stall);
+        tc_issue_two(sm, ts.taddr & 0xFFFFu, 0, m, (t0 + 7) >> 3, ts.stall);
         ts.pend_next = ts.pend_rest = true;
         // w = L xi, here and in the panels behind the barrier that others wait at
         // (rows past T are zero rows in the head columns)
@@ -476,7 +487,7 @@ __device__ __forceinline__ int hi_tc_step(HITCShared& sm, TCState& ts, const Cha
             if (!head && warp > pn) tc_put_operand<8>(sm, tid, A, !valid);
             tc::fence_async_smem();
             __syncthreads();
-            if (tid == 0) tc_issue_two(sm, ts.taddr, c0 + 32, m, 4, ts.stall);
+            tc_issue_two(sm, ts.taddr & 0xFFFFu, c0 + 32, m, 4, ts.stall);
             ts.pend_next = ts.pend_rest = true;
         } else {
             __syncthreads();       // every read of sm.lt done before the next step writes it
