@@ -333,9 +333,9 @@ bd_status bd_kernel_times(bd_ctx* ctx, double* ms, int64_t* launches);
  * seeded at each window end, their summed sensitivity injected into the
  * parent's adjoint at the window start. The parameter gradients accumulate
  * in the integration precision over blocks of 16 steps and in float64
- * across blocks, lanes and warps. Work buffers (about (K + 1) M and
- * min(K / window_steps, fit) (window_steps + 1) x all-slot bonds states) are
- * allocated on the first call and kept. Synchronises the stream. */
+ * across blocks, lanes and warps. Work buffers (2 K M parent states, and for
+ * as many windows as fill the GPU, at most K / window_steps, window_steps + 1
+ * states of every replica) are allocated on the first call and kept. Synchronises the stream. */
 bd_status bd_adjoint(bd_ctx* ctx, const double* grad_rsf, const double* grad_log_surv,
                      double* grad_params);
 

@@ -128,7 +128,7 @@ struct bd_ctx {
     std::vector<AdjChain> h_adj;
     std::vector<ItemDev> h_adj_items;
     std::vector<AdjClass> adj_classes;
-    int64_t adj_stride = 0, rep_batch = 0;
+    int64_t adj_stride = 0, rep_batch = 0, rep_window = 0;   // mu row; windows a batch; elements of a window's states
     AdjChain* d_adj = nullptr;
     ItemDev* d_adj_items = nullptr;
     void* d_seg[2] = {nullptr, nullptr};    // parent segments, alternating
@@ -1303,21 +1303,30 @@ bd_status adj_plan(bd_ctx* ctx)
 }
 
 // Work buffers of bd_adjoint: a K-row parent segment, the parent adjoint,
-// and replica-window batches sized to a quarter of the free device memory
+// and replica-window batches of at most a quarter of the free device memory
 // (between 1 and 32 GiB).
+constexpr int64_t kAdjPlaces = 3;
 bd_status adj_buffers(bd_ctx* ctx)
 {
     if (ctx->d_seg[0]) return BD_OK;
     const int64_t K = ctx->cfg.checkpoint_steps, S = ctx->cfg.window_steps, M = ctx->M;
-    const size_t per_window = ctx->tsize * 3 * (size_t)ctx->state_bonds * (size_t)(S + 1) +
-                              sizeof(double) * 3 * 2 * (size_t)ctx->adj_stride;
+    ctx->rep_window = 0;
+    for (const AdjClass& ac : ctx->adj_classes) ctx->rep_window += (int64_t)ac.item_count * (S + 1) * 96 * ac.L;
+    const size_t per_window = ctx->tsize * (size_t)ctx->rep_window + sizeof(double) * 3 * 2 * (size_t)ctx->adj_stride;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
         free_b = 0;
     }
     const int64_t budget = std::min<int64_t>(32ll << 30, std::max<int64_t>(1ll << 30, (int64_t)(free_b / 4)));
-    ctx->rep_batch = std::max<int64_t>(1, std::min<int64_t>({K / S, 65535, budget / (int64_t)per_window}));
+    // windows a batch: enough warps for kAdjPlaces rounds of the GPU (16 warps an
+    // SM), no more: a larger batch runs no faster and its memory costs its owner
+    // time (256 chains x 32 replicas of 200 beads, a training step of 10 windows:
+    // 31.3 ms with one window or two a batch, 34.8 with three, 36.4 with the five
+    // that fit: freeing their 11 GB takes 9 ms)
+    const int64_t fill = (kAdjPlaces * 16 * (int64_t)ctx->n_sm + (int64_t)ctx->h_adj_items.size() - 1) /
+                         std::max<int64_t>(1, (int64_t)ctx->h_adj_items.size());
+    ctx->rep_batch = std::max<int64_t>(1, std::min<int64_t>({K / S, 65535, fill, budget / (int64_t)per_window}));
     BD_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->adj_stream, cudaStreamNonBlocking));
     cudaEvent_t* evs[] = {&ctx->ev_init, &ctx->ev_done, &ctx->ev_win[0], &ctx->ev_win[1],
                           &ctx->ev_mu_free[0], &ctx->ev_mu_free[1], &ctx->ev_seg_free[0],
@@ -1330,8 +1339,7 @@ bd_status adj_buffers(bd_ctx* ctx)
                                                         (size_t)ctx->rep_batch)) != BD_OK) return s;
     }
     if ((s = dalloc(ctx, &ctx->d_lamP, ctx->tsize * 3 * (size_t)M)) != BD_OK) return s;
-    if ((s = dalloc(ctx, &ctx->d_repbuf, ctx->tsize * 3 * (size_t)ctx->state_bonds * (size_t)(S + 1) *
-                                             (size_t)ctx->rep_batch)) != BD_OK) return s;
+    if ((s = dalloc(ctx, &ctx->d_repbuf, ctx->tsize * (size_t)ctx->rep_window * (size_t)ctx->rep_batch)) != BD_OK) return s;
     if ((s = dalloc(ctx, (void**)&ctx->d_gls, sizeof(double) * (size_t)ctx->cfg.n_chains)) != BD_OK) return s;
     return dalloc(ctx, (void**)&ctx->d_grad, sizeof(double) * 3 * (size_t)ctx->cfg.n_chains);
 }
@@ -1895,7 +1903,7 @@ bd_status bd_adjoint(bd_ctx* ctx, const double* grad_rsf, const double* grad_log
         a.adj = ctx->d_adj;
         a.ckpt = ctx->d_ckpt;
         a.repbuf = ctx->d_repbuf;
-        a.state_bonds = ctx->state_bonds;
+        a.rep_window = ctx->rep_window;
         a.lamP = ctx->d_lamP;
         a.G = ctx->d_G;
         a.mu_stride = ctx->adj_stride;
@@ -1933,11 +1941,13 @@ bd_status bd_adjoint(bd_ctx* ctx, const double* grad_rsf, const double* grad_log
                 a.mu_w0 = b0;
                 a.w_batch0 = b0;
                 BD_CUDA(ctx, cudaStreamWaitEvent(S0, ctx->ev_mu_free[mb], 0));
+                a.rep_base = 0;
                 for (const AdjClass& ac : ctx->adj_classes) {
                     a.items = ctx->d_adj_items + ac.item_begin;
                     a.n_items = ac.item_count;
                     const dim3 grid((unsigned)((ac.item_count + per_cta - 1) / per_cta), (unsigned)(b1 - b0));
                     if ((s = adj_launch(ctx, ADJ_REPLICA_WINDOW, ac.L, grid, &a, S0)) != BD_OK) return s;
+                    a.rep_base += (int64_t)ac.item_count * (S + 1) * 96 * ac.L;
                 }
                 BD_CUDA(ctx, cudaEventRecord(ctx->ev_win[mb], S0));
                 BD_CUDA(ctx, cudaStreamWaitEvent(S1, ctx->ev_win[mb], 0));

@@ -169,8 +169,9 @@ struct AdjParams {
     int64_t ckpt_index;        // checkpoint the parent recompute starts from
     void* segbuf;              // T [K + 1][M][3] parent states of the segment
     int64_t seg_t0;            // step of segbuf row 0
-    void* repbuf;              // T [batch][S + 1][state_bonds][3] replica states
-    int64_t state_bonds;
+    void* repbuf;              // T [batch][items][S + 1][3 L][32] replica states (keep_state)
+    int64_t rep_window;        // elements of one window of repbuf
+    int64_t rep_base;          // first element of this launch's items in a window
     int64_t w_batch0;          // replica kernel: window of blockIdx.y = 0
     void* lamP;                // T [M][3] parent adjoint carried between segments
     const double* G;           // [w_hi - w_lo][M] dObjective / dRSF, row 0 = window w_lo
