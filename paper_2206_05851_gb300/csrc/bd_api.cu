@@ -320,7 +320,7 @@ void split_replicas(int c, int R, int per_warp, int v, std::vector<ItemDev>& ite
 // items, and the cost is their issue work per useful bead-step. Collapsed
 // chains (harmonic springs) take the collapsed-chain variants, the others
 // the rest; the tile and layout hints apply to the latter.
-VariantChoice choose_variant(const bd_ctx* ctx, int N, int R, bool collapsed, bool hi)
+VariantChoice choose_variant(const bd_ctx* ctx, int N, int R, bool collapsed, bool hi, bool shortest)
 {
     const bd_config& cfg = ctx->cfg;
     if (hi) return {kHIBase + (N > kHISmallBeadsHost ? 1 : 0), 1, R, 0.0};   // one CTA per replica
@@ -341,7 +341,8 @@ VariantChoice choose_variant(const bd_ctx* ctx, int N, int R, bool collapsed, bo
         if (G > 32) continue;
         const int per_warp = (paired ? 2 : 1) * (32 / G);
         const int groups = item_count(R, per_warp, v);
-        const double cost = groups * ctx->var_cost[v] / ((double)R * N);
+        // `shortest`: the shortest step of a warp, whatever it holds
+        const double cost = shortest ? ctx->var_cost[v] + 1e-6 * groups : groups * ctx->var_cost[v] / ((double)R * N);
         if (cost < best.cost - 1e-12) best = {v, per_warp, groups, cost};
     }
     return best;
@@ -462,10 +463,33 @@ bd_status validate(bd_ctx* ctx, const bd_config* cfg)
     return BD_OK;
 }
 
+// Whether the batch is so small that every warp of a launch has an SM
+// sub-partition (float32: half of one) to itself even on the tiles with the
+// shortest step, over as many windows as one chunk can hold: then a step's
+// length is all that counts, and more lanes a replica make it shorter (24
+// uneven chains of 3 to 61 beads, a window of 25 steps: 50 us a launch on the
+// tiles that use the fewest warps, 27 us on these; 4 float64 chains of 100
+// beads, 100 steps: 1.09 and 0.32 ms).
+bool shortest_steps(const bd_ctx* ctx)
+{
+    const bd_config& cfg = ctx->cfg;
+    const int64_t W = std::max<int64_t>(1, std::min<int64_t>(64, cfg.max_windows));
+    const int64_t most = (ctx->f64 ? 4 : 8) * (int64_t)ctx->n_sm;
+    int64_t items = 0;
+    for (int c = 0; c < cfg.n_chains && items * W <= most; ++c) {
+        const bd_chain_desc& d = ctx->chains[c];
+        if (d.hi_a > 0) continue;
+        items += choose_variant(ctx, d.n_beads, d.n_replicas, d.spring == BD_SPRING_HARMONIC || d.spring == BD_SPRING_VWF,
+                                false, true).groups;
+    }
+    return items * W <= most;
+}
+
 bd_status plan(bd_ctx* ctx)
 {
     const bd_config& cfg = ctx->cfg;
     const int C = cfg.n_chains;
+    const bool shortest = shortest_steps(ctx);
     ctx->h_chains.resize(C);
     int64_t bead = 0, slot_bead = 0, bond = 0, spr = 0, part = 0, rep = 0, bpart = 0;
     std::vector<ItemDev> items;
@@ -476,7 +500,7 @@ bd_status plan(bd_ctx* ctx)
         ChainDev& h = ctx->h_chains[c];
         const bool collapsed = d.spring == BD_SPRING_HARMONIC || d.spring == BD_SPRING_VWF;
         const bool hi = d.hi_a > 0;
-        const VariantChoice vc = choose_variant(ctx, d.n_beads, d.n_replicas, collapsed, hi);
+        const VariantChoice vc = choose_variant(ctx, d.n_beads, d.n_replicas, collapsed, hi, shortest);
         if (!vc.variant)
             return fail(ctx, BD_E_INVALID, "chain %d: no step variant fits N=%d", c, d.n_beads);
         h.N = d.n_beads; h.R = d.n_replicas; h.n_groups = vc.groups; h.spring = d.spring;

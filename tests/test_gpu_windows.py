@@ -93,3 +93,24 @@ def test_float64_noise_tables_outlive_the_context_that_filled_them():
     c.step(20)
     np.testing.assert_array_equal(c.positions(True), want[4])
     c.close()
+
+
+@pytest.mark.parametrize("batch", ["one", "dumbbell", "uneven", "collapsed"])
+def test_small_batches_take_the_shortest_step(batch):
+    """A batch that leaves every warp an SM sub-partition of its own runs on the tiles with the shortest step that fit its
+    chains; float32 results do not depend on the tile."""
+    chains = BATCHES[batch]
+    wl = I.custom(chains, 4e-5 if batch == "collapsed" else 1e-3, 6, 12)
+    got = []
+    for hints in ({}, {"lanes_hint": 16, "layout_hint": 1}):
+        ctx = bdra.Context(chains, wl.dt, 6, 11, I.initial_positions(wl, seed=5), max_windows=2,
+                           stream=torch.cuda.current_stream().cuda_stream, **hints)
+        if not hints:
+            for c, v in zip(chains, ctx.plan()[0]):
+                tiles = (202, 204, 205, 207, 216) if batch == "collapsed" else (4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16)
+                assert v == next(t for t in tiles if -(-c.n_beads // (t % 100)) <= 32)
+        ctx.step(12)
+        got.append((ctx.replica_average(1), ctx.positions(True)))
+        ctx.close()
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
