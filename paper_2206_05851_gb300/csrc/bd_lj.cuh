@@ -18,7 +18,18 @@ namespace bdra {
 
 template <typename T, bool FAST> struct Rsqrt {
     static __device__ __forceinline__ T rsqrt(T x) { return ::rsqrt(x); }
-    static __device__ __forceinline__ T rcp(T x) { return T(1) / x; }
+    // two Newton-Raphson steps y <- y + y (1 - x y) on the hardware's
+    // approximation (relative error below 2^-20, so 2^-40, then rounding: within
+    // an ulp or so), for squared distances, which are neither infinite nor
+    // subnormal. A division takes twice the float64 instructions: 32 collapsed
+    // chains x 20 replicas of 50 beads, 50 steps, 5.42 ms with it, 5.00 ms without.
+    static __device__ __forceinline__ T rcp(T x)
+    {
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"((double)x));
+        y = fma(y, fma(-(double)x, y, 1.0), y);
+        return (T)fma(y, fma(-(double)x, y, 1.0), y);
+    }
 };
 template <> struct Rsqrt<float, true> {
     static __device__ __forceinline__ float rsqrt(float x)
