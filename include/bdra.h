@@ -181,9 +181,10 @@ typedef struct {
     int64_t step;             /* global step of the parents */
     int64_t windows_done;     /* completed sampling windows */
     int64_t overextensions;   /* FENE-floor applications so far, all slots */
-    int64_t device_bytes;     /* device memory held by the context */
+    int64_t device_bytes;     /* device memory held by the context (without the 24 MB of
+                                 noise tables that a device's float64 contexts share) */
     int64_t kernel_launches;  /* CUDA kernels launched by this context so far */
-    int32_t n_launch_classes; /* kernel launches per bd_step chunk */
+    int32_t n_launch_classes; /* parent and replica kernels of the plan */
     int32_t precision;
 } bd_info;
 
@@ -204,8 +205,10 @@ bd_status bd_spawn_replicas(bd_ctx* ctx);
  * spawning replicas at each window start, sampling RSF (replicas, once at the
  * window end) and TSF/ISF (parent, every step), and updating the ISF
  * criteria. The work runs in chunks of up to 64 windows, each one launch of
- * a CUDA graph (parent kernels, then one persistent replica kernel per step
- * variant), asynchronous on the context's stream. BD_E_CAPACITY if the run
+ * a CUDA graph (parent kernels and one persistent replica kernel per step
+ * variant; the windows of a launch may run side by side, and replicas beside
+ * the parents where they do not need them yet), asynchronous on the context's
+ * stream. BD_E_CAPACITY if the run
  * would pass max_windows windows. n_steps = 0 is a no-op. */
 bd_status bd_step(bd_ctx* ctx, int64_t n_steps);
 

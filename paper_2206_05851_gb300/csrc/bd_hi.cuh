@@ -12,9 +12,10 @@
 //
 // One CTA integrates one slot (parent or replica) of a chain of N <= 64
 // beads, its positions (centre-of-mass frame) in shared memory. The 3N x 3N
-// tensor is held as 4 x 4 tiles of its lower triangle in the registers of
-// the CTA's threads (tile t of the column-major lower order belongs to
-// thread t mod kHIThreads). Per step:
+// tensor is held as 4 x 4 tiles of its lower triangle, in float32 in the
+// registers of the CTA's threads (tile t of the column-major lower order
+// belongs to thread t mod kHIThreads), in float64 in shared memory (HIEngine64,
+// below). Per step, in the register form:
 //   - bead forces (springs; Lennard-Jones split over four threads a bead) and
 //     bead normals;
 //   - the tensor, one 3 x 3 bead block per thread at a time, into a

@@ -11,7 +11,8 @@
 //   parent_kernel  advances every parent, writes its conformation at each
 //                  window end (the "halted parent" that the next window's
 //                  replicas copy; bd_set_positions writes the first), and
-//                  samples it every step (ISF criteria, TSF sums);
+//                  samples it every step (ISF criteria, TSF sums); few
+//                  parents run on parent_block_kernel instead;
 //   replica_kernel one CTA per (chain, replica group) evolves the replicas
 //                  window after window: spawn from the parent snapshot, S
 //                  steps, one force sample per replica at the window end,
