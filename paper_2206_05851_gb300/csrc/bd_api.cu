@@ -1690,13 +1690,20 @@ bd_status bd_detect_events(bd_ctx* ctx, bd_event* out, int64_t capacity, int64_t
         if (s != BD_OK) return s;
         dst = (bd_event*)ctx->d_io;
     }
-    ctx->launches += 3;
-    BD_CUDA(ctx, run_events(ctx->d_chains, ctx->d_spring_chain, ctx->M, ctx->d_first_thr,
-                            ctx->d_first_bell, ctx->d_evt_scratch, ctx->d_dev_err, dst, capacity, ctx->stream));
     const bool ldev = log_surv && is_device_ptr(log_surv);
-    if (ldev) {          // before the one wait of this call
+    if (ctx->M <= small_events()) {
         ++ctx->launches;
-        BD_CUDA(ctx, run_log_survival(ctx->d_chains, ctx->cfg.n_chains, ctx->M, ctx->d_lam, log_surv, ctx->stream));
+        BD_CUDA(ctx, run_events_small(ctx->d_chains, ctx->d_spring_chain, ctx->M, ctx->cfg.n_chains, ctx->d_first_thr,
+                                      ctx->d_first_bell, ctx->d_lam, ctx->d_dev_err, ctx->d_evt_scratch + nblk, dst,
+                                      capacity, ldev ? log_surv : nullptr, ctx->stream));
+    } else {
+        ctx->launches += 3;
+        BD_CUDA(ctx, run_events(ctx->d_chains, ctx->d_spring_chain, ctx->M, ctx->d_first_thr,
+                                ctx->d_first_bell, ctx->d_evt_scratch, ctx->d_dev_err, dst, capacity, ctx->stream));
+        if (ldev) {          // before the one wait of this call
+            ++ctx->launches;
+            BD_CUDA(ctx, run_log_survival(ctx->d_chains, ctx->cfg.n_chains, ctx->M, ctx->d_lam, log_surv, ctx->stream));
+        }
     }
     int64_t seen[2] = {0, 0};        // events, device error bits
     BD_CUDA(ctx, cudaMemcpyAsync(seen, ctx->d_evt_scratch + nblk, sizeof(seen), cudaMemcpyDeviceToHost, ctx->stream));

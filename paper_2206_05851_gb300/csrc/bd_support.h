@@ -27,6 +27,13 @@ int64_t event_blocks(int64_t M);
 cudaError_t run_events(const ChainDev* chains, const int32_t* spring_chain, int64_t M,
                        const int64_t* first_thr, const int64_t* first_bell, int64_t* block_scratch,
                        const int32_t* dev_err, bd_event* out, int64_t capacity, cudaStream_t st);
+// Count, list and (log_surv not NULL: device) log-survival in one CTA, for M <=
+// small_events(); seen: event count and error word.
+int64_t small_events();
+cudaError_t run_events_small(const ChainDev* chains, const int32_t* spring_chain, int64_t M, int n_chains,
+                             const int64_t* first_thr, const int64_t* first_bell, const double* lam,
+                             const int32_t* dev_err, int64_t* seen, bd_event* out, int64_t capacity,
+                             double* log_surv, cudaStream_t st);
 cudaError_t run_log_survival(const ChainDev* chains, int n_chains, int64_t M, const double* lam,
                              double* out, cudaStream_t st);
 cudaError_t run_adj_seed(const ChainDev* chains, const int32_t* spring_chain, int64_t M,

@@ -114,3 +114,35 @@ def test_small_batches_take_the_shortest_step(batch):
         ctx.close()
     for a, b in zip(*got):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("beads", [(2,), (200, 57), (200, 58), (200, 59), (500, 500, 500, 500, 53), (500, 500, 500, 500, 54)])
+def test_event_list_and_survival_at_the_edges_of_the_one_cta_form(beads):
+    """M = 1, 255, 256, 257 and 2048 springs (one CTA), 2049 (block counts): the list equals the first-event arrays in its
+    documented order, the log-survival the hazards' sums."""
+    chains = [_fene(n, 3) for n in beads]
+    wl = I.custom(chains, 5e-3, 10, 60)
+    ctx = bdra.Context(chains, wl.dt, 10, 3, I.initial_positions(wl, seed=9), max_windows=6, thr_mask=7, bell_mask=7,
+                       stream=torch.cuda.current_stream().cuda_stream)
+    ctx.step(60)
+    ev, surv = ctx.events()
+    dev_list = torch.zeros((6 * ctx.M, 24), dtype=torch.uint8, device="cuda")
+    dev_surv = torch.zeros((len(chains), 3), dtype=torch.float64, device="cuda")
+    n = bdra.bd_detect_events(ctx.ptr, dev_list, 6 * ctx.M, dev_surv)
+    haz, thr, bell = ctx.kinetics()
+    ctx.close()
+    want, at = [], 0
+    for c, ch in enumerate(chains):
+        for i in range(ch.n_beads - 1):
+            for q in range(3):
+                want += [(c, i, q, k, int(a[q, at + i])) for k, a in ((0, thr), (1, bell)) if a[q, at + i] >= 0]
+        at += ch.n_beads - 1
+    assert [tuple(int(x) for x in e) for e in ev] == want and n == len(want)
+    np.testing.assert_array_equal(dev_list.cpu().numpy()[:n].reshape(-1).view(bdra.EVENT_DTYPE), ev)
+    assert len(beads) == 1 or want
+    at = 0
+    for c, ch in enumerate(chains):
+        s = -haz[:, at:at + ch.n_beads - 1].sum(axis=1)
+        np.testing.assert_allclose(surv[c], s, rtol=ch.n_beads * 2.0 ** -52)     # another order of the sum
+        at += ch.n_beads - 1
+    np.testing.assert_array_equal(dev_surv.cpu().numpy(), surv)
