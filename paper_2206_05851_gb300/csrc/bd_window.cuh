@@ -123,9 +123,9 @@ __device__ __forceinline__ void run_one_item_h(const ItemDev& it, const StepRang
     const T* snap = reinterpret_cast<const T*>(p.snap);
     T qx[L], qy[L], qz[L];
     // the replica's state where the launch starts inside a window, else the
-    // snapshot (read again by the loop: an unconditional load costs nothing, a
-    // branch around it 12 registers on the 4-spring tile); a part after the
-    // first never reads the state that the last one writes
+    // snapshot (one load from either place: a branch around it cost 12 registers
+    // on the 4-spring tile); a part after the first never reads the state that
+    // the last one writes
     load_bonds<T, L>(qx, qy, qz, rg.s_in != 0 ? state : snap + ((int64_t)(rg.w % p.win_ring) * p.M + ch.spr_off) * 3, lc);
 
     int floored = 0;
@@ -133,7 +133,7 @@ __device__ __forceinline__ void run_one_item_h(const ItemDev& it, const StepRang
     int w = rg.w;                                   // window index (< 2^31)
 #pragma unroll 1
     for (uint32_t t = rg.t0; t < rg.t1; ++t) {
-        if (s_in == 0)   // spawn: copy the halted parent (Sec. II)
+        if (s_in == 0 && t != rg.t0)   // spawn: copy the halted parent (Sec. II)
             load_bonds<T, L>(qx, qy, qz, snap + ((int64_t)(w % p.win_ring) * p.M + ch.spr_off) * 3, lc);
         if constexpr (LJ)
             floored += step_bonds_lj<T, L, FAST, TAB, H>(qx, qy, qz, lc, k, kl, sw < P, sw < P ? lane - sw * G : 0, G,

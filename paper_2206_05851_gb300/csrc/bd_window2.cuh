@@ -300,7 +300,7 @@ __device__ __forceinline__ void run_pair_item_k(const ItemDev& it, const StepRan
     int w = rg.w;                                   // window index (< 2^31)
 #pragma unroll 1
     for (uint32_t t = rg.t0; t < rg.t1; ++t) {
-        if (s_in == 0) {  // spawn both replicas from the halted parent (Sec. II)
+        if (s_in == 0 && t != rg.t0) {  // spawn both replicas from the halted parent (Sec. II)
             const float* src = snap + ((int64_t)(w % p.win_ring) * p.M + ch.spr_off) * 3;
 #pragma unroll
             for (int j = 0; j < L; ++j) {
