@@ -7,8 +7,11 @@ contiguous ranges, one per rank (one process per GPU), with no exchange
 during the integration. Each rank's context takes its range's first global
 chain index as ``chain_id_base``, so that its chains draw the noise of the
 whole workload: the union of the ranks' results is, bit for bit, the result
-of the whole workload in one context. The ranges are balanced by the cost of
-a chain, N (R + 1) slot-beads a step (parent and replicas).
+of the whole workload in one context (with the planner's own costs; ranks that
+call ``bd_autotune`` may measure other ones, and for chains whose sums follow the
+tile - collapsed chains, float64, the Eq. 5 diagnostics - agree to rounding).
+The ranges are balanced by the cost of a chain, N (R + 1) slot-beads a step
+(parent and replicas).
 
 The only collectives come after the integration: the event lists are
 gathered (each rank's list is in (chain, spring, criterion, kind) order and

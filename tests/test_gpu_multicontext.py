@@ -134,3 +134,51 @@ def test_range_matches_the_oracle_with_global_chain_ids():
     ctx, g0 = _run(sub, p0, bdra.BD_PREC_FP64, 0)
     ctx.close()
     assert not np.allclose(g0["rsf"], g["rsf"])
+
+
+def _batch(kind, n_sm):
+    """A workload that is a large batch in one piece and a small one in each of its two halves: by the work items of a launch
+    (up to 8 warps an SM in float32, 4 in float64, are few) or by the warps of parents (5 an SM)."""
+    if kind == "collapsed":
+        ch = I.collapsed_chain(50)
+        ch.f_c, ch.k0, ch.dx = 30.0, 5.0, 0.1
+        return [ch] * (2 * (8 * n_sm // 50))
+    if kind == "parents":
+        fene = [I.Chain(n_beads=n, n_replicas=2, spring=I.SPRING_FENE, flow=I.FLOW_SHEAR, b=40.0, rate=0.5, f_c=3.0, k0=0.5, dx=0.5)
+                for n in (50, 30)]
+        return fene * (2 * (245 * n_sm // 100))
+    ch = I.Chain(n_beads=100, n_replicas=8, spring=I.SPRING_FENE, flow=I.FLOW_PLANAR, b=60.0, rate=0.2, f_c=3.0, k0=0.5, dx=0.5)
+    return [ch] * (2 * ((4 if kind == "fp64" else 8) * n_sm // 8))
+
+
+@pytest.mark.parametrize("kind,prec,flags", [("collapsed", bdra.BD_PREC_FP32, 0), ("collapsed", bdra.BD_PREC_FP64, 0),
+                                             ("fp64", bdra.BD_PREC_FP64, 0), ("fp32", bdra.BD_PREC_FP32, 0),
+                                             ("fp32", bdra.BD_PREC_FP32, bdra.BD_FLAG_CONFORMATION),
+                                             ("parents", bdra.BD_PREC_FP32, 0), ("parents", bdra.BD_PREC_FP64, 0)])
+def test_a_large_workload_equals_its_small_halves(kind, prec, flags):
+    """The launch shapes that depend on how much work a context has (tiles, parent kernel, windows side by side) leave every
+    result of a chain as it is: the halves of a large workload are small batches."""
+    import torch
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    chains = _batch(kind, n_sm)
+    if kind == "collapsed" and prec == bdra.BD_PREC_FP64:
+        chains = chains[:2 * (4 * n_sm // 50)]
+    dt = I.COLLAPSED_DT if kind == "collapsed" else DT
+    pos0 = I.initial_positions(I.custom(chains, dt, 20, 20), seed=4)
+    half = len(chains) // 2
+    beads = sum(c.n_beads for c in chains[:half])
+
+    def run(sub, p0, base):
+        ctx = bdra.Context(sub, dt, 20, SEED, p0, precision=prec, max_windows=1, thr_mask=7, bell_mask=7, flags=flags,
+                           stream=_stream(), chain_id_base=base)
+        ctx.step(20)
+        out = [ctx.replica_average(0), ctx.time_average(0), ctx.positions(True), *(a.T for a in ctx.kinetics()), ctx.events(6 * ctx.M)[1]]
+        if flags & bdra.BD_FLAG_CONFORMATION:
+            out += list(ctx.conformation(0))
+        ctx.close()
+        return out
+
+    whole = run(chains, pos0, 0)
+    a, b = run(chains[:half], pos0[:beads], 0), run(chains[half:], pos0[beads:], half)
+    for w, x, y in zip(whole, a, b, strict=True):
+        np.testing.assert_array_equal(np.concatenate([x, y]), w)
