@@ -1,0 +1,72 @@
+"""The integrator's float64 device functions against what they stand for: the FENE floor taken by the bits of s against the
+comparison it replaces."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2206_05851_gb300 import bdra
+from paper_2206_05851_gb300 import build as B
+from paper_2206_05851_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def dev():
+    import torch
+    lib = B.build()
+    torch.cuda.init()
+    out = os.path.join(HERE, "_build", f"device_checks_{os.getpid()}.so")
+    os.makedirs(os.path.dirname(out), exist_ok=True)
+    r = subprocess.run([B._nvcc(), *B.ARCH, *B.COMMON, "-fmad=false", "-I", B.CSRC, "-shared", "-o", out,
+                        os.path.join(HERE, "device_checks.cu"), lib, "-Xlinker", f"-rpath={os.path.dirname(lib)}"],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    yield ctypes.CDLL(out)
+    os.unlink(out)
+
+
+def _p(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+@pytest.mark.parametrize("Hinvb", [1.0, 0.25, 0.0])
+def test_fene_floor_by_bits_is_the_comparison(dev, Hinvb):
+    """s < smin is floored and counted; a NaN s (of either sign) takes smin, as fmax does, and is not counted. The bond
+    lengths are dyadic, so that s is exact and the host's expressions give the same bits."""
+    H, smin, nan, inf = 1.5, 2.0 ** -9, np.nan, np.inf
+    u = np.array([[62, 12, 10], [63, 12, 10], [62, 12, 9], [64, 0, 0], [128, 0, 0], [0, 0, 0], [1, 0, 0], [124, 24, 20],
+                  [126, 24, 20]]) / 64.0           # first: s = smin exactly with Hinvb = 1; [124, 24, 20] with 1/4
+    odd = np.array([[nan, 0, 0], [-nan, 0, 0], [0, nan, 1], [inf, 0, 0], [-inf, 1, 0], [inf, nan, 0], [1e200, 0, 0]])
+    r = np.random.default_rng(4)
+    q = np.ascontiguousarray(np.concatenate([u, odd, r.integers(-160, 160, size=(1000, 3)) / 128.0]))
+    c, fl = np.zeros(len(q)), np.zeros(len(q), dtype=np.int32)
+    assert dev.check_spring(ctypes.c_int64(len(q)), _p(q), ctypes.c_double(H), ctypes.c_double(Hinvb), ctypes.c_double(smin),
+                            _p(c), _p(fl)) == 0
+    with np.errstate(all="ignore"):
+        s = 1.0 - Hinvb * (q * q).sum(axis=1)
+        want = H / np.fmax(s, smin)
+    np.testing.assert_array_equal(fl, (s < smin).astype(np.int32))
+    np.testing.assert_array_equal(c, want)
+    assert np.isnan(s).any() and (fl[:len(u)].any() or Hinvb == 0.0)
+
+
+@pytest.mark.parametrize("prec", [bdra.BD_PREC_FP64, bdra.BD_PREC_FP32])
+def test_bonds_that_are_not_numbers_count_no_overextension(prec):
+    """A NaN bead in a FENE chain; a Hooke chain whose squared bond overflows (s = 1 - 0 inf); a sound chain beside them."""
+    import torch
+    chains = [I.Chain(n_beads=12, n_replicas=3, spring=k, flow=I.FLOW_SHEAR, b=30.0, rate=0.1)
+              for k in (I.SPRING_FENE, I.SPRING_HOOKE, I.SPRING_FENE)]
+    pos = I.initial_positions(I.custom(chains, 1e-4, 5, 10), seed=3)
+    pos[4], pos[16, 1] = np.nan, 1e200
+    ctx = bdra.Context(chains, 1e-4, 5, 1, pos, precision=prec, max_windows=2, stream=torch.cuda.current_stream().cuda_stream)
+    ctx.step(10)
+    n, end = ctx.info().overextensions, ctx.positions()
+    ctx.close()
+    assert np.isnan(end[:12]).any() and np.isfinite(end[24:]).all()
+    assert n == 0
