@@ -18,17 +18,26 @@ namespace bdra {
 
 template <typename T, bool FAST> struct Rsqrt {
     static __device__ __forceinline__ T rsqrt(T x) { return ::rsqrt(x); }
-    // two Newton-Raphson steps y <- y + y (1 - x y) on the hardware's
-    // approximation (relative error below 2^-20, so 2^-40, then rounding: within
-    // an ulp or so), for squared distances, which are neither infinite nor
-    // subnormal. A division takes twice the float64 instructions: 32 collapsed
-    // chains x 20 replicas of 50 beads, 50 steps, 5.42 ms with it, 5.00 ms without.
+    // Two Newton-Raphson steps y <- y + y (1 - x y) on the hardware's
+    // approximation: its relative error, below 2^-20, is squared to 2^-40 and
+    // below 2^-79, so the last multiply-add rounds a value that is right far
+    // beyond the last place, and the result is 1 / x or a neighbour of it (over
+    // 400,000 random arguments, the powers of two, their neighbours and the
+    // separations of lj_far: at most one unit in the last place). Zero and
+    // infinite arguments, for which the steps would give NaN, keep the
+    // approximation's infinity or zero; so do squared distances outside 2^-1022
+    // .. 2^1022, whose reciprocals a division gives to the last subnormal. A division
+    // takes twice the float64 instructions: 32 collapsed chains x 20 replicas
+    // of 50 beads, 50 steps, 5.42 ms with it, 5.00 ms without.
     static __device__ __forceinline__ T rcp(T x)
     {
         double y;
         asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"((double)x));
-        y = fma(y, fma(-(double)x, y, 1.0), y);
-        return (T)fma(y, fma(-(double)x, y, 1.0), y);
+        const double y1 = fma(y, fma(-(double)x, y, 1.0), y);
+        const double y2 = fma(y1, fma(-(double)x, y1, 1.0), y1);
+        // neither zero nor infinite: the exponent field of y is 1 .. 2046
+        const unsigned e = (unsigned)__double2hiint(y) & 0x7ff00000u;
+        return (T)(e - 0x00100000u < 0x7fe00000u ? y2 : y);
     }
 };
 template <> struct Rsqrt<float, true> {

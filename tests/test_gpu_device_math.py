@@ -1,5 +1,5 @@
 """The integrator's float64 device functions against what they stand for: the FENE floor taken by the bits of s against the
-comparison it replaces."""
+comparison it replaces, the reciprocal of the pair forces against the division."""
 import ctypes
 import os
 import subprocess
@@ -70,3 +70,22 @@ def test_bonds_that_are_not_numbers_count_no_overextension(prec):
     ctx.close()
     assert np.isnan(end[:12]).any() and np.isfinite(end[24:]).all()
     assert n == 0
+
+
+def test_reciprocal_of_pair_forces(dev):
+    """Within one unit in the last place of 1 / x: two Newton-Raphson steps square a relative error of 2^-20 twice, so the last
+    multiply-add rounds a value within 2^-53 (2^-26) of the reciprocal, and 1 / x is its correctly rounded neighbour. Zero and
+    infinite squared distances (coincident and overflowing beads) as the division."""
+    r = np.random.default_rng(8)
+    rnd = np.ldexp(r.uniform(1.0, 2.0, 400_000), r.integers(-1020, 1020, 400_000))
+    two = np.ldexp(1.0, np.arange(-1020, 1020))
+    far = (1e12 * np.arange(1, 514)) ** 2
+    x = np.concatenate([rnd, two, np.nextafter(two, 0.0), np.nextafter(two, np.inf), far, [1e30, 1e36]])
+    x = np.ascontiguousarray(np.concatenate([x, -x[:1000], [0.0, -0.0, np.inf, -np.inf]]))
+    y = np.zeros(len(x))
+    assert dev.check_recip(ctypes.c_int64(len(x)), _p(x), _p(y)) == 0
+    with np.errstate(divide="ignore"):
+        want = 1.0 / x
+    np.testing.assert_array_equal(y[-4:], want[-4:])
+    ulps = np.abs(y[:-4].view(np.int64) - want[:-4].view(np.int64))
+    assert ulps.max() <= 1
