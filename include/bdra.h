@@ -51,11 +51,11 @@
  *     the last three. The Exp(1) thresholds of the Bell first-passage test:
  *     counter (spring, 1 << 24, criterion, chain), E = -ln((x0 + 1/2) 2^-32).
  *     The noise therefore does not depend on the launch shape, and a chain's
- *     results not on the other chains of its context: the tile and the split
- *     into work items follow from its own N and R, except where the results
- *     are the same bits on every tile (float32 Hooke and FENE chains without
- *     BD_FLAG_CONFORMATION). bd_autotune may change the tile of any chain and
- *     with it the order of sums (last bits) of the others.
+ *     results not on the other chains of its context: the tile and the order
+ *     of sums follow from its own N and R, except where the results are the
+ *     same bits on every tile (Hooke and FENE chains without
+ *     BD_FLAG_CONFORMATION). bd_autotune may change the tile of any chain, and
+ *     with it the order of those sums (last bits).
  */
 #ifndef BDRA_H
 #define BDRA_H

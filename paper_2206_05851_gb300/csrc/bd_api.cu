@@ -465,25 +465,28 @@ bd_status validate(bd_ctx* ctx, const bd_config* cfg)
 
 // Whether chains of this law may take a tile that depends on the rest of the
 // batch. A workload split over contexts has the whole run's results bit for
-// bit, so only where they do not depend on the tile: float32 Hooke and FENE
-// chains without Eq. 5 (their steps round the same on every tile, and the
-// float64 sums of their float32 tensions are exact in any order, unless the R
-// tensions of a spring span more than 2^29 / R). Collapsed chains sum positions and
-// pair forces, Eq. 5 the beads and float64 runs the replicas in the tile's order.
-bool tile_is_free(const bd_ctx* ctx, bool collapsed) { return !ctx->f64 && !ctx->conf && !collapsed; }
+// bit, so only where they do not depend on the tile: Hooke and FENE chains
+// without Eq. 5. Their steps round the same on every tile; the float64 sums of
+// float32 tensions are exact in any order (unless the R tensions of a spring
+// span more than 2^29 / R), those of float64 tensions are formed in the order
+// of the chain's own tile (ChainDev::own_per_warp). Collapsed chains sum
+// positions and pair forces, Eq. 5 the beads, in the tile's order.
+bool tile_is_free(const bd_ctx* ctx, bool collapsed) { return !ctx->conf && !collapsed; }
 
-// Whether the batch is so small that every warp of a launch has half an SM
-// sub-partition to itself even on the tiles with the shortest step, over as
-// many windows as one chunk can hold (of the max_windows that the context has
-// room for): then a step's length is all that counts, and more lanes a replica
-// make it shorter (24 uneven chains of 3 to 61 beads, a window of 25 steps: 50 us
-// a launch on the tiles that use the fewest warps, 27 us on these).
+// Whether the batch is so small that every warp of a launch has an SM
+// sub-partition (float32: half of one) to itself even on the tiles with the
+// shortest step, over as many windows as one chunk can hold (of the max_windows
+// that the context has room for): then a step's length is all that counts, and
+// more lanes a replica make it shorter (24 uneven chains of 3 to 61 beads, a
+// window of 25 steps: 50 us a launch on the tiles that use the fewest warps, 27
+// us on these; 4 float64 chains of 100 beads, 8 replicas, a pass of 100 steps:
+// 2.11 and 0.65 ms).
 bool shortest_steps(const bd_ctx* ctx)
 {
     const bd_config& cfg = ctx->cfg;
     if (!tile_is_free(ctx, false)) return false;
     const int64_t W = std::max<int64_t>(1, std::min<int64_t>(64, cfg.max_windows));
-    const int64_t most = 8 * (int64_t)ctx->n_sm;
+    const int64_t most = (ctx->f64 ? 4 : 8) * (int64_t)ctx->n_sm;
     int64_t items = 0;
     for (int c = 0; c < cfg.n_chains && items * W <= most; ++c) {
         const bd_chain_desc& d = ctx->chains[c];
@@ -509,7 +512,9 @@ bd_status plan(bd_ctx* ctx)
         ChainDev& h = ctx->h_chains[c];
         const bool collapsed = d.spring == BD_SPRING_HARMONIC || d.spring == BD_SPRING_VWF;
         const bool hi = d.hi_a > 0;
-        const VariantChoice vc = choose_variant(ctx, d.n_beads, d.n_replicas, collapsed, hi, shortest && tile_is_free(ctx, collapsed));
+        const VariantChoice own = choose_variant(ctx, d.n_beads, d.n_replicas, collapsed, hi, false);
+        const VariantChoice vc = shortest && tile_is_free(ctx, collapsed) && !hi
+                                     ? choose_variant(ctx, d.n_beads, d.n_replicas, collapsed, hi, true) : own;
         if (!vc.variant)
             return fail(ctx, BD_E_INVALID, "chain %d: no step variant fits N=%d", c, d.n_beads);
         h.N = d.n_beads; h.R = d.n_replicas; h.n_groups = vc.groups; h.spring = d.spring;
@@ -544,7 +549,7 @@ bd_status plan(bd_ctx* ctx)
         h.f32[6] = (float)(h.kzz * cfg.dt);
         h.f32[7] = (float)(h.kxz * cfg.dt);
         h.f32[8] = (float)cfg.s_min;
-        h.f32_pad = 0.0f;
+        h.own_per_warp = ctx->f64 && vc.variant != own.variant ? own.per_warp : 0;
         const int nb = d.n_beads - 1;
         // warp items: replicas split as evenly as the warp capacity allows
         split_replicas(c, d.n_replicas, vc.per_warp, vc.variant, items);
@@ -558,7 +563,7 @@ bd_status plan(bd_ctx* ctx)
         slot_bead += (int64_t)(d.n_replicas + 1) * d.n_beads;
         bond += (int64_t)(d.n_replicas + 1) * nb;
         spr += nb;
-        part += (int64_t)vc.groups * nb;
+        part += (int64_t)(h.own_per_warp > 0 ? d.n_replicas : vc.groups) * nb;
         rep += d.n_replicas;
         bpart += (int64_t)vc.groups * d.n_beads;
     }

@@ -37,7 +37,11 @@ struct ChainDev {
     // sqrt(2 D dt) times the fast normals' sign, kappa_xx dt, kappa_yy dt,
     // kappa_zz dt, kappa_xz dt, s_min
     float f32[9];
-    float f32_pad;
+    // 0: the partial row has one entry a spring and work item (n_groups). Else
+    // (float64 small batches, whose tile depends on the batch) one a spring and
+    // replica, and the fold adds them as the work items of the chain's own
+    // tile, of up to this many replicas each, would.
+    int32_t own_per_warp;
 };
 
 // One warp's work: replicas rep_begin + 1 + stride s, s = 0 .. rep_count-1,

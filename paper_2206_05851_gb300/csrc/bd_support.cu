@@ -119,13 +119,29 @@ positions_kernel(const ChainDev* chains, const int64_t* pair_off, int n_chains, 
 }
 
 // RSF of window w, spring i of a chain: the chain's per-group partial sums
-// (ring slot w % ring) in group order, over R.
+// (ring slot w % ring) in group order, over R. Of per-replica rows
+// (ChainDev::own_per_warp) the sums are formed here, in the groups that
+// split_replicas (bd_api.cu) makes of up to own_per_warp replicas: the odd
+// replicas, then the even ones, each as evenly as they go; one by one for 1.
 __device__ __forceinline__ double rsf_of(const ChainDev& ch, const double* part, int64_t part_stride,
                                          int64_t slot, int64_t i)
 {
     const int nb = ch.N - 1;
     const double* row = part + slot * part_stride + ch.part_off + i;
     double acc = 0.0;
+    if (ch.own_per_warp > 0) {
+        const int step = ch.own_per_warp == 1 ? 1 : 2;
+        for (int h = 0; h < step; ++h) {
+            const int n = (ch.R - h + step - 1) / step, groups = (n + ch.own_per_warp - 1) / ch.own_per_warp;
+            int r = h;
+            for (int g = 0; g < groups; ++g) {
+                double a = 0.0;
+                for (int k = n / groups + (g < n % groups ? 1 : 0); k > 0; --k, r += step) a += row[(int64_t)r * nb];
+                acc += a;
+            }
+        }
+        return acc / (double)ch.R;
+    }
 #pragma unroll 8
     for (int g = 0; g < ch.n_groups; ++g) acc += row[(int64_t)g * nb];
     return acc / (double)ch.R;

@@ -89,6 +89,17 @@ __device__ __forceinline__ void warp_window_sum(const T* wsm, int nb, int count,
     __syncwarp();
 }
 
+// The same samples a row a replica (ChainDev::own_per_warp); prow: replica 0's.
+template <typename T>
+__device__ __forceinline__ void warp_window_rows(const T* wsm, int nb, const ItemDev& it, double* prow)
+{
+    __syncwarp();
+    for (int s = 0; s < it.rep_count; ++s)
+        for (int i = (int)(threadIdx.x & 31); i < nb; i += 32)
+            prow[(int64_t)(it.rep_begin + it.stride * s) * nb + i] = (double)wsm[s * nb + i];
+    __syncwarp();
+}
+
 // With TAB, ptab is this warp's table of 32 L bead parts of the Philox
 // counter (filled here for the item's chain). CONF compiles in the Eq. 5
 // window-end diagnostics (used when BD_FLAG_CONFORMATION is set); without it
@@ -153,8 +164,9 @@ __device__ __forceinline__ void run_one_item_h(const ItemDev& it, const StepRang
                                : spring_tension<T, FAST>(qx[j], qy[j], qz[j], k.H, k.Hinvb, k.smin);
                 }
             }
-            warp_window_sum<T>(wsm, nb, it.rep_count,
-                               p.part_hist + (int64_t)(w % p.win_ring) * p.part_stride + ch.part_off + (int64_t)it.group * nb);
+            double* prow = p.part_hist + (int64_t)(w % p.win_ring) * p.part_stride + ch.part_off;
+            if (sizeof(T) == 8 && !LJ && !CONF && ch.own_per_warp > 0) warp_window_rows<T>(wsm, nb, it, prow);
+            else warp_window_sum<T>(wsm, nb, it.rep_count, prow + (int64_t)it.group * nb);
             if (CONF && (p.flags & BD_FLAG_CONFORMATION)) {
                 T* mine = conf + (sw < P ? sw : 0) * nb * 3;
                 store_bonds<T, L>(qx, qy, qz, mine, lc);

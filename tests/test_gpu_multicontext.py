@@ -147,12 +147,16 @@ def _batch(kind, n_sm):
         fene = [I.Chain(n_beads=n, n_replicas=2, spring=I.SPRING_FENE, flow=I.FLOW_SHEAR, b=40.0, rate=0.5, f_c=3.0, k0=0.5, dx=0.5)
                 for n in (50, 30)]
         return fene * (2 * (245 * n_sm // 100))
+    if kind == "shapes":       # 60 items on the shortest tiles; other splits of odd and even replicas on the chains' own
+        return [I.Chain(n_beads=n, n_replicas=r, spring=I.SPRING_FENE, flow=I.FLOW_PLANAR, b=60.0, rate=0.05, f_c=3.0, k0=0.5, dx=0.5)
+                for n, r in ((100, 9), (64, 8), (33, 13), (20, 31), (10, 50), (200, 5), (500, 3), (2, 4))] * (2 * (4 * n_sm // 60))
     ch = I.Chain(n_beads=100, n_replicas=8, spring=I.SPRING_FENE, flow=I.FLOW_PLANAR, b=60.0, rate=0.2, f_c=3.0, k0=0.5, dx=0.5)
     return [ch] * (2 * ((4 if kind == "fp64" else 8) * n_sm // 8))
 
 
 @pytest.mark.parametrize("kind,prec,flags", [("collapsed", bdra.BD_PREC_FP32, 0), ("collapsed", bdra.BD_PREC_FP64, 0),
-                                             ("fp64", bdra.BD_PREC_FP64, 0), ("fp32", bdra.BD_PREC_FP32, 0),
+                                             ("fp64", bdra.BD_PREC_FP64, 0), ("shapes", bdra.BD_PREC_FP64, 0),
+                                             ("fp32", bdra.BD_PREC_FP32, 0),
                                              ("fp32", bdra.BD_PREC_FP32, bdra.BD_FLAG_CONFORMATION),
                                              ("parents", bdra.BD_PREC_FP32, 0), ("parents", bdra.BD_PREC_FP64, 0)])
 def test_a_large_workload_equals_its_small_halves(kind, prec, flags):
