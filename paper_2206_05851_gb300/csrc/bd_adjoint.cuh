@@ -122,30 +122,62 @@ __device__ __forceinline__ void load_lane(const T* q, const LaneCtx& lc, T (&x)[
     }
 }
 
-// The lane's L bonds of one stored step of a replica window. Only the lane that
-// wrote a state reads it back, so its place is free: component 3 j + d of all
-// lanes side by side, 128 bytes a warp instruction. (In bond order a lane's 3 L
-// values lay together and each of the 21 stores of a 7-spring tile touched a
-// sector per lane, eight times the sectors that the data fill: 256 chains x 32
-// replicas of 200 beads, 10 windows of 100 steps: 21.3 ms, now 17.4 ms.)
-template <typename T, int L>
-__device__ __forceinline__ void keep_state(T* row, int lane, const T (&x)[L], const T (&y)[L], const T (&z)[L])
-{
-#pragma unroll
-    for (int j = 0; j < L; ++j) {
-        row[(3 * j + 0) * 32 + lane] = x[j];
-        row[(3 * j + 1) * 32 + lane] = y[j];
-        row[(3 * j + 2) * 32 + lane] = z[j];
+// Where a lane keeps the bonds of its replica in the steps of a window. Only the
+// lane that wrote a state reads it back, so its place is free: a lane with bonds
+// has a column, 32 columns make a sheet [S + 1][3 L][32], and value 3 j + d
+// (component d of bond j) of a step is 32 values from the next, so the
+// offsets are the instructions' own and a warp's values lie in one or two
+// lines. (In bond order a lane's 3 L values lay together and each of the 21
+// stores of a 7-spring tile touched a sector per lane, eight times the sectors
+// that the data fill: 256 chains x 32 replicas of 200 beads, 10 windows of 100
+// steps: 21.3 ms, now 17.4 ms.) The columns of the lanes at work follow one another
+// through the items, whatever part of a warp they fill: the states take the room of
+// the bonds, up to the L - rem < L that the last lane of a replica lacks. PACK, for
+// chains of few lanes, where that would show (2 beads: four times): the last lanes
+// have columns of their own, each shared by L / rem of equal rem.
+template <int L, bool PACK> struct Kept {
+    int rem, lanes, m;        // bonds of a replica's last lane; columns a replica takes by itself; last lanes in a shared one
+    __device__ __forceinline__ Kept(int nb, int G)
+    {
+        rem = nb - (G - 1) * L;
+        lanes = G - (PACK || rem == 0 ? 1 : 0);
+        m = PACK && rem > 0 ? L / rem : 1;
     }
+    // element of step 0, value 0 of the lane `seg` of replica k = 0 .. R - 1, in the sheets of the chain's class
+    __device__ __forceinline__ int64_t place(const AdjChain& ac, int k, int seg, int S) const
+    {
+        int64_t c = ac.keep_off + (int64_t)k * lanes + seg;
+        int shared_row = 0;
+        if (PACK && seg == lanes) {
+            const int64_t i = ac.tail_first + k;
+            c = ac.tail_off + i / m;
+            shared_row = (int)(i % m) * rem * 3;
+        }
+        return ((c >> 5) * (S + 1) * (3 * L) + shared_row) * 32 + (c & 31);
+    }
+};
+
+template <typename T, int L, bool PACK>
+__device__ __forceinline__ void keep_state(T* row, bool mine, const LaneCtx& lc, const T (&x)[L], const T (&y)[L], const T (&z)[L])
+{
+#pragma unroll
+    for (int j = 0; j < L; ++j)
+        if (PACK ? j < lc.nv : mine) {
+            row[(3 * j + 0) * 32] = x[j];
+            row[(3 * j + 1) * 32] = y[j];
+            row[(3 * j + 2) * 32] = z[j];
+        }
 }
-template <typename T, int L>
-__device__ __forceinline__ void take_state(const T* row, int lane, T (&x)[L], T (&y)[L], T (&z)[L])
+// Lanes without a column read that of the warp's first lane; they use nothing of it.
+template <typename T, int L, bool PACK>
+__device__ __forceinline__ void take_state(const T* row, const LaneCtx& lc, T (&x)[L], T (&y)[L], T (&z)[L])
 {
 #pragma unroll
     for (int j = 0; j < L; ++j) {
-        x[j] = row[(3 * j + 0) * 32 + lane];
-        y[j] = row[(3 * j + 1) * 32 + lane];
-        z[j] = row[(3 * j + 2) * 32 + lane];
+        const bool held = !PACK || j < lc.nv;
+        x[j] = held ? row[(3 * j + 0) * 32] : T(0);
+        y[j] = held ? row[(3 * j + 1) * 32] : T(0);
+        z[j] = held ? row[(3 * j + 2) * 32] : T(0);
     }
 }
 
@@ -258,10 +290,10 @@ __global__ void __launch_bounds__(kAdjThreads) adj_parent_recompute_kernel(const
 // Replica windows w = w_batch0 + blockIdx.y (one warp = one work item):
 // recompute the S steps from the parent state at the window start (segbuf),
 // keeping every state; seed lambda = (G_w / R) grad f at the window end; S
-// adjoint steps back; then mu_w of the item's replicas. Each lane reads back
-// only the bonds it wrote itself, so the two sweeps need no synchronisation.
+// adjoint steps back; then mu_w of the item's replicas. Each lane uses only
+// the bonds it wrote itself.
 // ---------------------------------------------------------------------------
-template <typename T, int L, bool FAST>
+template <typename T, int L, bool FAST, bool PACK>
 __global__ void __launch_bounds__(kAdjThreads) adj_replica_window_kernel(const AdjParams a)
 {
     __shared__ uint4 tab_all[kAdjThreads / 32][32 * L];    // split-Philox bead parts per warp
@@ -282,8 +314,11 @@ __global__ void __launch_bounds__(kAdjThreads) adj_replica_window_kernel(const A
     const LaneCtx lc = make_lane(seg, G, L, lane, nb, active, key, (uint32_t)it.chain + p.chain_base);
     const int64_t w = a.w_batch0 + blockIdx.y;
     const int64_t tw = w * p.S;
-    const int64_t row = 96 * L;                             // one step of the item's part of repbuf
-    T* rb = reinterpret_cast<T*>(a.repbuf) + (int64_t)blockIdx.y * a.rep_window + a.rep_base + (int64_t)gw * (p.S + 1) * row;
+    const int64_t row = 96 * L;                             // one step of a sheet
+    const Kept<L, PACK> kept(nb, G);
+    const bool mine = active && (PACK || seg < kept.lanes);
+    T* rb = reinterpret_cast<T*>(a.repbuf) + (int64_t)blockIdx.y * a.rep_window + a.rep_base +
+            kept.place(ac, it.rep_begin + (mine ? sw : 0), mine ? seg : 0, p.S);
 
     // forward: spawn from the parent at tw, S steps, every state kept
     {
@@ -296,13 +331,14 @@ __global__ void __launch_bounds__(kAdjThreads) adj_replica_window_kernel(const A
         T qx[L], qy[L], qz[L];
         load_bonds<T, L>(qx, qy, qz,
                          reinterpret_cast<const T*>(a.segbuf) + ((tw - a.seg_t0) * p.M + ch.spr_off) * 3, lc);
-        keep_state<T, L>(rb, lane, qx, qy, qz);
+        keep_state<T, L, PACK>(rb, mine, lc, qx, qy, qz);
 #pragma unroll 1
         for (int s = 0; s < p.S; ++s) {
             step_bonds<T, L, FAST, true>(qx, qy, qz, lc, k, (uint32_t)(tw + s), p, tab);
-            keep_state<T, L>(rb + (int64_t)(s + 1) * row, lane, qx, qy, qz);
+            keep_state<T, L, PACK>(rb + (int64_t)(s + 1) * row, mine, lc, qx, qy, qz);
         }
     }
+    __syncwarp();              // lanes without a column read the first lane's
 
     // backward
     AdjConst<T> k;
@@ -312,7 +348,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_replica_window_kernel(const A
     T lx[L], ly[L], lz[L];
     {
         T ex[L], ey[L], ez[L];
-        take_state<T, L>(rb + (int64_t)p.S * row, lane, ex, ey, ez);
+        take_state<T, L, PACK>(rb + (int64_t)p.S * row, lc, ex, ey, ez);
         const double* Gw = a.G + (w - a.w_lo) * p.M + ch.spr_off;
         const double invR = 1.0 / (double)ch.R;
 #pragma unroll
@@ -336,11 +372,11 @@ __global__ void __launch_bounds__(kAdjThreads) adj_replica_window_kernel(const A
     }
     // states are loaded one step ahead of the sweep that uses them
     T qx[L], qy[L], qz[L];
-    take_state<T, L>(rb + (int64_t)(p.S - 1) * row, lane, qx, qy, qz);
+    take_state<T, L, PACK>(rb + (int64_t)(p.S - 1) * row, lc, qx, qy, qz);
 #pragma unroll 1
     for (int s = p.S - 1; s >= 0; --s) {
         T nx[L], ny[L], nz[L];
-        take_state<T, L>(rb + (int64_t)(s > 0 ? s - 1 : 0) * row, lane, nx, ny, nz);
+        take_state<T, L, PACK>(rb + (int64_t)(s > 0 ? s - 1 : 0) * row, lc, nx, ny, nz);
         adjoint_step<T, L>(qx, qy, qz, lx, ly, lz, lc, k, ga.part);
         ga.tick();
 #pragma unroll

@@ -28,10 +28,13 @@ const void* adj_func_f32(int kind, int L)
         break;
     case ADJ_REPLICA_WINDOW:
         switch (L) {
-#define X(l) case l: return (const void*)adj_replica_window_kernel<float, l, true>;
+#define X(l) case l: return (const void*)adj_replica_window_kernel<float, l, true, false>;
             BD_ADJ_REPLICA_TILES(X)
 #undef X
         }
+        break;
+    case ADJ_REPLICA_WINDOW_PACKED:
+        if (L == kAdjTiles[0]) return (const void*)adj_replica_window_kernel<float, kAdjTiles[0], true, true>;
         break;
     }
     return nullptr;

@@ -28,10 +28,13 @@ const void* adj_func_f64(int kind, int L)
         break;
     case ADJ_REPLICA_WINDOW:
         switch (L) {
-#define X(l) case l: return (const void*)adj_replica_window_kernel<double, l, false>;
+#define X(l) case l: return (const void*)adj_replica_window_kernel<double, l, false, false>;
             BD_ADJ_REPLICA_TILES(X)
 #undef X
         }
+        break;
+    case ADJ_REPLICA_WINDOW_PACKED:
+        if (L == kAdjTiles[0]) return (const void*)adj_replica_window_kernel<double, kAdjTiles[0], false, true>;
         break;
     }
     return nullptr;

@@ -41,7 +41,9 @@ constexpr int kParentHIKey = 2000;   // planner key of the parents with hydrodyn
 
 struct AdjClass {      // one adjoint replica-window launch: the work items of one tile
     int L;
+    bool pack;         // the storage of short chains (Kept)
     int item_begin, item_count;
+    int64_t columns;   // of stored states
 };
 
 }  // namespace
@@ -1293,7 +1295,9 @@ bd_status adj_plan(bd_ctx* ctx)
     const bd_config& cfg = ctx->cfg;
     const int C = cfg.n_chains;
     ctx->h_adj.assign(C, AdjChain{});
-    std::vector<std::pair<int, ItemDev>> items;
+    std::vector<std::pair<std::pair<int, bool>, ItemDev>> items;
+    std::map<std::pair<int, bool>, int64_t> columns;
+    std::map<int, int64_t> tails;       // packed: last lanes by rem, whose columns follow (tail_at)
     int64_t part = 0;
     for (int c = 0; c < C; ++c) {
         const bd_chain_desc& d = ctx->chains[c];
@@ -1307,6 +1311,15 @@ bd_status adj_plan(bd_ctx* ctx)
         a.part_off = part;
         a.n_groups = groups;
         a.pad = 0;
+        // the columns of its replicas (Kept): one a lane with bonds, packed: one a full lane
+        const std::pair<int, bool> cls(L, L == kAdjTiles[0] && G <= kAdjPackLanes);
+        const int rem = d.n_beads - 1 - (G - 1) * L;
+        a.keep_off = columns[cls];
+        columns[cls] += (int64_t)d.n_replicas * (G - (cls.second || rem == 0 ? 1 : 0));
+        if (cls.second && rem > 0) {
+            a.tail_first = tails[rem];
+            tails[rem] += d.n_replicas;
+        }
         a.khat[0] = a.khat[1] = a.khat[2] = a.khat[3] = 0.0;
         switch (d.flow) {
         case BD_FLOW_SHEAR: a.khat[3] = 1.0; break;
@@ -1317,19 +1330,31 @@ bd_status adj_plan(bd_ctx* ctx)
         int begin = 0;
         for (int g = 0; g < groups; ++g) {
             const int cnt = d.n_replicas / groups + (g < d.n_replicas % groups ? 1 : 0);
-            items.push_back({L, ItemDev{c, g, begin, cnt, L, 1}});
+            items.push_back({cls, ItemDev{c, g, begin, cnt, L, 1}});
             begin += cnt;
         }
         part += (int64_t)groups * (d.n_beads - 1);
     }
     ctx->adj_stride = part;
+    std::map<int, int64_t> tail_at;
+    for (const auto& t : tails) {       // L / rem of them a column
+        int64_t& cols = columns[{kAdjTiles[0], true}];
+        tail_at[t.first] = cols;
+        const int m = kAdjTiles[0] / t.first;
+        cols += (t.second + m - 1) / m;
+    }
+    for (int c = 0; c < C; ++c) {
+        const int N = ctx->chains[c].n_beads, L = kAdjTiles[0], G = (N + L - 1) / L;
+        if (G <= kAdjPackLanes && (N - 1) % L) ctx->h_adj[c].tail_off = tail_at[(N - 1) % L];
+    }
     std::stable_sort(items.begin(), items.end(),
-                     [](const std::pair<int, ItemDev>& x, const std::pair<int, ItemDev>& y) { return x.first < y.first; });
+                     [](const auto& x, const auto& y) { return x.first < y.first; });
     ctx->h_adj_items.clear();
     ctx->adj_classes.clear();
     for (size_t k = 0; k < items.size(); ++k) {
-        if (ctx->adj_classes.empty() || ctx->adj_classes.back().L != items[k].first)
-            ctx->adj_classes.push_back(AdjClass{items[k].first, (int)k, 0});
+        const std::pair<int, bool>& cls = items[k].first;
+        if (ctx->adj_classes.empty() || ctx->adj_classes.back().L != cls.first || ctx->adj_classes.back().pack != cls.second)
+            ctx->adj_classes.push_back(AdjClass{cls.first, cls.second, (int)k, 0, columns[cls]});
         ctx->adj_classes.back().item_count++;
         ctx->h_adj_items.push_back(items[k].second);
     }
@@ -1344,12 +1369,17 @@ bd_status adj_plan(bd_ctx* ctx)
 // and replica-window batches of at most a quarter of the free device memory
 // (between 1 and 32 GiB).
 constexpr int64_t kAdjPlaces = 3;
+// Values of one window's stored states of a class, in whole sheets of 32 columns.
+int64_t adj_class_states(const bd_ctx* ctx, const AdjClass& ac)
+{
+    return (ac.columns + 31) / 32 * ((int64_t)ctx->cfg.window_steps + 1) * 96 * ac.L;
+}
 bd_status adj_buffers(bd_ctx* ctx)
 {
     if (ctx->d_seg[0]) return BD_OK;
     const int64_t K = ctx->cfg.checkpoint_steps, S = ctx->cfg.window_steps, M = ctx->M;
     ctx->rep_window = 0;
-    for (const AdjClass& ac : ctx->adj_classes) ctx->rep_window += (int64_t)ac.item_count * (S + 1) * 96 * ac.L;
+    for (const AdjClass& ac : ctx->adj_classes) ctx->rep_window += adj_class_states(ctx, ac);
     const size_t per_window = ctx->tsize * (size_t)ctx->rep_window + sizeof(double) * 3 * 2 * (size_t)ctx->adj_stride;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
@@ -1991,8 +2021,9 @@ bd_status bd_adjoint(bd_ctx* ctx, const double* grad_rsf, const double* grad_log
                     a.items = ctx->d_adj_items + ac.item_begin;
                     a.n_items = ac.item_count;
                     const dim3 grid((unsigned)((ac.item_count + per_cta - 1) / per_cta), (unsigned)(b1 - b0));
-                    if ((s = adj_launch(ctx, ADJ_REPLICA_WINDOW, ac.L, grid, &a, S0)) != BD_OK) return s;
-                    a.rep_base += (int64_t)ac.item_count * (S + 1) * 96 * ac.L;
+                    if ((s = adj_launch(ctx, ac.pack ? ADJ_REPLICA_WINDOW_PACKED : ADJ_REPLICA_WINDOW, ac.L, grid, &a, S0)) != BD_OK)
+                        return s;
+                    a.rep_base += adj_class_states(ctx, ac);
                 }
                 BD_CUDA(ctx, cudaEventRecord(ctx->ev_win[mb], S0));
                 BD_CUDA(ctx, cudaStreamWaitEvent(S1, ctx->ev_win[mb], 0));

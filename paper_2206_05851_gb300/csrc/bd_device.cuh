@@ -157,6 +157,9 @@ __device__ __forceinline__ StepRange item_range(const StepParams& p, int part)
 // Adjoint (bd_adjoint.cuh): per chain, for the adjoint only.
 struct AdjChain {
     int64_t part_off;    // first entry of this chain's group 0 in a mu row
+    // columns of its replicas' stored states (Kept) in the sheets of its class: the first
+    // one; packed: the first of the last lanes with its rem, its own first one among these
+    int64_t keep_off, tail_off, tail_first;
     int32_t n_groups;    // adjoint replica groups (warp items) of the chain
     int32_t pad;
     double khat[4];      // kappa / rate: xx, yy, zz, xz
@@ -173,9 +176,9 @@ struct AdjParams {
     int64_t ckpt_index;        // checkpoint the parent recompute starts from
     void* segbuf;              // T [K + 1][M][3] parent states of the segment
     int64_t seg_t0;            // step of segbuf row 0
-    void* repbuf;              // T [batch][items][S + 1][3 L][32] replica states (keep_state)
+    void* repbuf;              // T [batch][classes][sheets][S + 1][3 L][32] replica states (Kept)
     int64_t rep_window;        // elements of one window of repbuf
-    int64_t rep_base;          // first element of this launch's items in a window
+    int64_t rep_base;          // first element of this launch's class in a window
     int64_t w_batch0;          // replica kernel: window of blockIdx.y = 0
     void* lamP;                // T [M][3] parent adjoint carried between segments
     const double* G;           // [w_hi - w_lo][M] dObjective / dRSF, row 0 = window w_lo

@@ -87,10 +87,13 @@ size_t persist_smem_f64(int variant);
 
 // Adjoint kernels (bd_adjoint.cuh), launched with kAdjThreads threads (bd_device.cuh): the
 // parent kernels exist for every tile of kTiles, the replica-window kernel
-// for the tiles of kAdjTiles.
-enum { ADJ_PARENT_RECOMPUTE = 0, ADJ_REPLICA_WINDOW = 1, ADJ_PARENT_BACKWARD = 2 };
-static const int kAdjTiles[] = {4, 7, 16};
-static const int kNumAdjTiles = 3;
+// for the tiles of kAdjTiles, with packed states (chains of at most
+// kAdjPackLanes lanes) for the first. From nine lanes on, the bonds that a
+// replica's last lane lacks are less than a tenth of its own.
+enum { ADJ_PARENT_RECOMPUTE = 0, ADJ_REPLICA_WINDOW = 1, ADJ_PARENT_BACKWARD = 2, ADJ_REPLICA_WINDOW_PACKED = 3 };
+constexpr int kAdjTiles[] = {4, 7, 16};
+constexpr int kNumAdjTiles = 3;
+constexpr int kAdjPackLanes = 8;
 const void* adj_func_f32(int kind, int L);
 const void* adj_func_f64(int kind, int L);
 

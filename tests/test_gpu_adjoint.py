@@ -331,3 +331,38 @@ def test_adjoint_workload_full_size_sampled_chains():
     want = oracle_grad(sub, r, dr, Gs, gls[sample], wl.dt, S_)
     assert so[-1] == Gs.shape[1]
     assert_close(got[sample], want, 1e-3, "adjoint workload")
+
+
+@pytest.mark.parametrize("prec,rtol", [(F64, 1e-10), (F32, 1e-3)])
+def test_adjoint_at_the_edges_of_its_tiles(prec, rtol):
+    """Chains whose last lane holds no spring, one, or all of them, in warps that are part filled (tiles of 4, 7 and 16 springs
+    a lane for up to 128, 224 and 512 beads), against the oracle's tangent."""
+    edges = [(2, 1), (2, 33), (4, 3), (5, 20), (8, 2), (9, 11), (128, 2), (129, 1), (134, 3), (224, 1), (225, 5), (497, 1), (512, 2)]
+    chains = [I.Chain(n_beads=n, n_replicas=r, spring=I.SPRING_FENE, flow=(I.FLOW_UNIAXIAL, I.FLOW_SHEAR, I.FLOW_PLANAR)[k % 3],
+                      b=40.0 + k, rate=0.3 / n, H=1.0 + 0.02 * k, k0=1e-3, dx=0.2) for k, (n, r) in enumerate(edges)]
+    S_, n = 7, 21
+    pos0 = I.initial_positions(I.custom(chains, DT, S_, n), seed=31)
+    G, gls = seeds(chains, n // S_, 8)
+    r, dr = O.rsf_tangent(chains, DT, S_, n, SEED, pos0, n_threads=4)
+    ctx = gpu_forward(chains, DT, S_, n, SEED, pos0, prec, S_)
+    got = ctx.adjoint(G, gls)
+    ctx.close()
+    assert_close(got, oracle_grad(chains, r, dr, G, gls, DT, S_), rtol, "edges")
+
+
+@pytest.mark.parametrize("n,R", [(2, 1), (5, 2), (20, 1), (130, 8), (300, 16)])
+def test_adjoint_stores_no_more_than_the_bonds_of_a_window(n, R):
+    """The states kept for one window take no more than the bonds of its slots (parents included), however few lanes of a warp
+    they fill."""
+    chains = [I.Chain(n_beads=n, n_replicas=R, spring=I.SPRING_FENE, flow=I.FLOW_SHEAR, b=40.0, rate=0.1)] * 256
+    S_, C, nb = 50, 256, n - 1
+    pos0 = I.initial_positions(I.custom(chains, DT, S_, S_), seed=5)
+    ctx = gpu_forward(chains, DT, S_, S_, SEED, pos0, F32, S_)
+    before = ctx.info().device_bytes
+    ctx.adjoint(np.ones((1, ctx.M)), np.ones(C))
+    grown = ctx.info().device_bytes - before
+    ctx.close()
+    M = C * nb
+    states = 12 * nb * C * (R + 1) * (S_ + 1)
+    segments, mu, rest = 2 * 12 * M * S_, 2 * 24 * M * R, 12 * M + 8 * M + 8 * C + 24 * C
+    assert grown <= states + segments + mu + rest
