@@ -19,14 +19,18 @@ using namespace bdra;
 
 namespace {
 
+struct LaunchShape {   // one replica launch (launch_shapes)
+    int grid, grid_y, block;
+    int32_t n_parts, win_per_part;
+    size_t conf_off;   // its warps' part of the stage's Eq. 5 scratch (elements)
+};
 struct VarClass {      // one persistent replica launch: the work items of one step variant
     int variant;
     int item_begin, item_count;
     int threads;
     int resident;      // CTAs of this kernel that the GPU holds
-    struct { int grid, grid_y, block; } shape[2];   // CTAs and threads of the chunk's two launches (chunk_shapes)
+    LaunchShape shape[2];   // of the chunk's two launches
     size_t smem;       // dynamic shared memory per CTA
-    size_t conf_off;   // its warps' part of the Eq. 5 scratch (elements)
 };
 struct ParClass {      // one parent-kernel launch: the parent warps of one tile
     int L, threads, grid;
@@ -86,8 +90,8 @@ struct bd_ctx {
     double* d_dpart = nullptr;          // [part_ring][bpart_stride][3]
     double* d_dbead = nullptr;          // [max_windows][sum N][3]
     double* d_rgz = nullptr;            // [max_windows][n_chains]
-    void* d_conf_scratch = nullptr;     // window-end bonds of the resident warps
-    size_t conf_elems = 0;              // of one replica launch; the two of a chunk may overlap
+    void* d_conf_scratch = nullptr;     // window-end bonds of the warps of a chunk's two replica stages
+    size_t conf_elems[2] = {0, 0};      // elements of each: the most that any number of windows takes
     double* d_tsf = nullptr;
     double* d_tsf_acc = nullptr;
     double* d_lam = nullptr;
@@ -499,6 +503,90 @@ bool shortest_steps(const bd_ctx* ctx)
     return items * W <= most;
 }
 
+// How many runs the W windows of a launch split into, given the work items
+// that run at the same time and how many of them the GPU holds at once
+// (places). With six units a place and more, splitting gains nothing: the
+// last warps run faster while others idle (1024 chains x 16 items, 6.7 a
+// place, 10 windows: 19.92 ms whole, 19.85 ms in 5 parts), and a warp pays
+// about 2 us to set a unit up and mixes the code of the two noise halves
+// (uneven chains, 10.5 a place: 8.2 ms whole, 8.6 ms split). Below that the
+// idle part of the last round shows: 4096 items, 1.7 a place, 4 windows:
+// 2.56 ms whole, 2.32 ms split. Chains with hydrodynamic interaction (a CTA a
+// unit, latency-bound: the last CTAs run no faster) take 24.
+int replica_parts(int64_t items, int64_t places, int64_t W, int64_t per_place)
+{
+    return (int)std::max<int64_t>(1, std::min(W, (per_place * places + items - 1) / items));
+}
+
+// The replica launches over W windows, each split into parts and its grid sized.
+// A launch with more units than the GPU holds warps takes every SM and goes
+// through its parts in order. Smaller ones (few chains, or one of many
+// variants) run side by side, each with its share of the SMs by work, every
+// part with CTAs of its own that hold as few warps as that share allows: a
+// warp alone on its SM sub-partition steps fastest (the float64 chain of 20
+// beads: 1.2 ms for ten windows side by side, 18.7 ms one after another).
+// Returns the Eq. 5 scratch that the launches take together (elements).
+size_t launch_shapes(const bd_ctx* ctx, int64_t W, std::vector<LaunchShape>& out)
+{
+    double total_work = 0.0;
+    int64_t total_units = 0, total_items = 0;
+    size_t conf = 0;
+    out.assign(ctx->var_classes.size(), LaunchShape{});
+    for (const VarClass& vc : ctx->var_classes)
+        if (!variant_hi(vc.variant)) total_items += vc.item_count;
+    for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
+        const VarClass& vc = ctx->var_classes[k];
+        const bool hi = variant_hi(vc.variant);
+        const int64_t warps = hi ? 1 : vc.threads / 32;
+        const int parts = replica_parts(hi ? vc.item_count : total_items, vc.resident * warps, W, hi ? 24 : 6);
+        LaunchShape& sh = out[k];
+        sh.win_per_part = (int32_t)((W + parts - 1) / parts);
+        sh.n_parts = (int32_t)((W + sh.win_per_part - 1) / sh.win_per_part);
+        if (hi) {
+            sh.grid = sh.n_parts * vc.item_count;
+            sh.grid_y = 1;
+            sh.block = vc.threads;
+            continue;
+        }
+        total_units += (int64_t)sh.n_parts * vc.item_count;
+        total_work += (double)sh.n_parts * vc.item_count * ctx->var_cost[vc.variant];
+    }
+    for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
+        const VarClass& vc = ctx->var_classes[k];
+        if (variant_hi(vc.variant)) continue;
+        LaunchShape& sh = out[k];
+        const int64_t most = vc.threads / 32, parts = sh.n_parts, units = parts * vc.item_count;
+        const double share = (double)units * ctx->var_cost[vc.variant] / total_work;
+        const int64_t ctas = total_units <= vc.resident ? units : std::max<int64_t>(1, (int64_t)(share * vc.resident));
+        int64_t warps = std::max<int64_t>(1, (units + ctas - 1) / ctas);
+        while (warps <= most && (vc.item_count + warps - 1) / warps * parts > ctas) ++warps;
+        if (warps <= most) {              // one unit a warp, every part its own CTAs
+            sh.grid = (int)((vc.item_count + warps - 1) / warps);
+            sh.grid_y = (int)parts;
+            sh.block = (int)(32 * warps);
+        } else {
+            sh.grid = (int)std::min<int64_t>((units + most - 1) / most, vc.resident);
+            sh.grid_y = 1;
+            sh.block = vc.threads;
+        }
+        sh.conf_off = conf;
+        if (ctx->conf) conf += (size_t)sh.grid * sh.grid_y * (vc.threads / 32) * 3 * variant_bonds(vc.variant);
+    }
+    return conf;
+}
+
+// Whether a chunk's parents run beside its replicas (chunk_stages).
+bool stages_overlap(const bd_ctx* ctx)
+{
+    int64_t items = 0, places = 0;
+    for (const VarClass& vc : ctx->var_classes) {
+        if (variant_hi(vc.variant)) return true;
+        items += vc.item_count;
+        places = std::max<int64_t>(places, (int64_t)vc.resident * (vc.threads / 32));
+    }
+    return 2 * items <= places;
+}
+
 bd_status plan(bd_ctx* ctx)
 {
     const bd_config& cfg = ctx->cfg;
@@ -581,10 +669,9 @@ bd_status plan(bd_ctx* ctx)
     const int threads = ctx->f64 ? persist_threads_f64() : persist_threads_f32();
     for (size_t k = 0; k < items.size(); ++k) {
         if (ctx->var_classes.empty() || ctx->var_classes.back().variant != items[k].variant)
-            ctx->var_classes.push_back(VarClass{items[k].variant, (int)k, 0, threads, 0, {}, 0, 0});
+            ctx->var_classes.push_back(VarClass{items[k].variant, (int)k, 0, threads, 0, {}, 0});
         ctx->var_classes.back().item_count++;
     }
-    ctx->conf_elems = 0;
     for (VarClass& vc : ctx->var_classes) {
         if (variant_hi(vc.variant)) {          // one CTA per replica
             cudaError_t e = ctx->f64 ? hi_prepare_f64() : hi_prepare_f32();
@@ -611,9 +698,6 @@ bd_status plan(bd_ctx* ctx)
             return fail(ctx, BD_E_CUDA, "occupancy of variant %d: %s", vc.variant, cudaGetErrorString(e));
         }
         vc.resident = per_sm * ctx->n_sm;
-        vc.conf_off = ctx->conf_elems;
-        if (ctx->conf)
-            ctx->conf_elems += (size_t)vc.resident * (threads / 32) * kConfSlots * 3 * variant_tile(vc.variant);
     }
     // parent launches: one per tile; warps pack parents of equal lane count
     // (parents of Hooke and FENE chains: of at most kParentBlockWarps warps an
@@ -666,6 +750,14 @@ bd_status plan(bd_ctx* ctx)
     // snapshot chunk: up to 64 windows, capped at ~512 MB
     const int64_t per_window = ctx->M * 3 * (int64_t)ctx->tsize;
     ctx->chunk_windows = std::max<int64_t>(1, std::min<int64_t>(64, (512ll << 20) / std::max<int64_t>(per_window, 1)));
+    // Eq. 5 scratch: the first stage holds one window, the second up to a
+    // chunk's (max_windows and an unfinished one)
+    std::vector<LaunchShape> shapes;
+    ctx->conf_elems[0] = stages_overlap(ctx) ? launch_shapes(ctx, 1, shapes) : 0;
+    ctx->conf_elems[1] = 0;
+    if (ctx->conf)
+        for (int64_t W = 1; W <= std::min(ctx->chunk_windows, cfg.max_windows + 1); ++W)
+            ctx->conf_elems[1] = std::max(ctx->conf_elems[1], launch_shapes(ctx, W, shapes));
     return BD_OK;
 }
 
@@ -712,68 +804,8 @@ StepParams base_params(const bd_ctx* ctx)
     return p;
 }
 
-// How many runs the W windows of a launch split into, given the work items
-// that run at the same time and how many of them the GPU holds at once
-// (places). With six units a place and more, splitting gains nothing: the
-// last warps run faster while others idle (1024 chains x 16 items, 6.7 a
-// place, 10 windows: 19.92 ms whole, 19.85 ms in 5 parts), and a warp pays
-// about 2 us to set a unit up and mixes the code of the two noise halves
-// (uneven chains, 10.5 a place: 8.2 ms whole, 8.6 ms split). Below that the
-// idle part of the last round shows: 4096 items, 1.7 a place, 4 windows:
-// 2.56 ms whole, 2.32 ms split. Chains with hydrodynamic interaction (a CTA a
-// unit, latency-bound: the last CTAs run no faster) take 24.
-int replica_parts(int64_t items, int64_t places, int64_t W, int64_t per_place)
-{
-    return (int)std::max<int64_t>(1, std::min(W, (per_place * places + items - 1) / items));
-}
-
 // Work-item counters of one replica launch, one a part.
 int64_t queue_len(const bd_ctx* ctx) { return ctx->chunk_windows; }
-
-// Splits every replica launch of steps [t0, t0 + n) and sizes its grid. A
-// launch with more units than the GPU holds warps takes every SM and goes
-// through its parts in order. Smaller ones (few chains, or one of many
-// variants) run side by side, each with its share of the SMs by work, every
-// part with CTAs of its own that hold as few warps as that share allows: a
-// warp alone on its SM sub-partition steps fastest (the float64 chain of 20
-// beads: 1.2 ms for ten windows side by side, 18.7 ms one after another).
-void chunk_shapes(bd_ctx* ctx, int stage, int64_t t0, int64_t n, std::vector<StepParams>& rp)
-{
-    const int64_t S = ctx->cfg.window_steps;
-    const int64_t W = std::max<int64_t>(1, (t0 + n + S - 1) / S - t0 / S);
-    double total_work = 0.0;
-    int64_t total_units = 0, total_items = 0;
-    for (const VarClass& vc : ctx->var_classes)
-        if (!variant_hi(vc.variant)) total_items += vc.item_count;
-    for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
-        VarClass& vc = ctx->var_classes[k];
-        const bool hi = variant_hi(vc.variant);
-        const int64_t warps = hi ? 1 : vc.threads / 32;
-        const int parts = replica_parts(hi ? vc.item_count : total_items, vc.resident * warps, W, hi ? 24 : 6);
-        rp[k].win_per_part = (int32_t)((W + parts - 1) / parts);
-        rp[k].n_parts = (int32_t)((W + rp[k].win_per_part - 1) / rp[k].win_per_part);
-        if (hi) {
-            vc.shape[stage] = {rp[k].n_parts * vc.item_count, 1, vc.threads};
-            continue;
-        }
-        total_units += (int64_t)rp[k].n_parts * vc.item_count;
-        total_work += (double)rp[k].n_parts * vc.item_count * ctx->var_cost[vc.variant];
-    }
-    for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
-        VarClass& vc = ctx->var_classes[k];
-        if (variant_hi(vc.variant)) continue;
-        const int64_t most = vc.threads / 32, parts = rp[k].n_parts, units = parts * vc.item_count;
-        const double share = (double)units * ctx->var_cost[vc.variant] / total_work;
-        const int64_t ctas = total_units <= vc.resident ? units : std::max<int64_t>(1, (int64_t)(share * vc.resident));
-        int64_t warps = std::max<int64_t>(1, (units + ctas - 1) / ctas);
-        while (warps <= most && (vc.item_count + warps - 1) / warps * parts > ctas) ++warps;
-        if (warps <= most) {              // one unit a warp, every part its own CTAs
-            vc.shape[stage] = {(int)((vc.item_count + warps - 1) / warps), (int)parts, (int)(32 * warps)};
-        } else {
-            vc.shape[stage] = {(int)std::min<int64_t>((units + most - 1) / most, vc.resident), 1, vc.threads};
-        }
-    }
-}
 
 // One chunk as up to two parent and two replica launches.
 struct Stage { int64_t t0, n; bool on, store; };
@@ -793,15 +825,8 @@ struct ChunkStages { Stage par[2], rep[2]; };
 ChunkStages chunk_stages(const bd_ctx* ctx, int64_t t0, int64_t n)
 {
     const int64_t S = ctx->cfg.window_steps, W = (n + S - 1) / S;
-    int64_t items = 0, places = 0;
-    bool hi = false;
-    for (const VarClass& vc : ctx->var_classes) {
-        if (variant_hi(vc.variant)) { hi = true; continue; }
-        items += vc.item_count;
-        places = std::max<int64_t>(places, (int64_t)vc.resident * (vc.threads / 32));
-    }
     ChunkStages c;
-    if (ctx->timing || t0 % S != 0 || !(hi || 2 * items <= places)) {
+    if (ctx->timing || t0 % S != 0 || !stages_overlap(ctx)) {
         c.par[0] = {t0, n, true, true};
         c.par[1] = {t0, 0, false, false};
         c.rep[0] = {t0, 0, false, false};
@@ -836,14 +861,20 @@ void replica_params(bd_ctx* ctx, int stage, const Stage& st, std::vector<StepPar
     p.t0 = st.t0; p.n_steps = st.n;
     p.store_state = st.store;
     rp.assign(ctx->var_classes.size(), p);
+    const int64_t S = ctx->cfg.window_steps;
+    std::vector<LaunchShape> shapes;
+    launch_shapes(ctx, std::max<int64_t>(1, (st.t0 + st.n + S - 1) / S - st.t0 / S), shapes);
     for (size_t k = 0; k < ctx->var_classes.size(); ++k) {
-        const VarClass& vc = ctx->var_classes[k];
+        VarClass& vc = ctx->var_classes[k];
+        vc.shape[stage] = shapes[k];
         rp[k].items = ctx->d_items + vc.item_begin;
         rp[k].n_items = vc.item_count;
+        rp[k].n_parts = shapes[k].n_parts;
+        rp[k].win_per_part = shapes[k].win_per_part;
         rp[k].queue = ctx->d_queue + (stage * ctx->var_classes.size() + k) * queue_len(ctx);
-        if (ctx->conf) rp[k].conf_scratch = (char*)ctx->d_conf_scratch + (stage * ctx->conf_elems + vc.conf_off) * ctx->tsize;
+        if (ctx->conf)
+            rp[k].conf_scratch = (char*)ctx->d_conf_scratch + ((stage ? ctx->conf_elems[0] : 0) + shapes[k].conf_off) * ctx->tsize;
     }
-    chunk_shapes(ctx, stage, st.t0, st.n, rp);
 }
 
 cudaKernelNodeParams parent_node(const bd_ctx* ctx, size_t k, StepParams* pk, void** args)
@@ -1255,7 +1286,7 @@ bd_status replan(bd_ctx* ctx)
     const size_t old_items = ctx->h_items.size();
     const int64_t old_part = ctx->part_stride;
     const int64_t old_bpart = ctx->bpart_stride;
-    const size_t old_conf = ctx->conf_elems;
+    const size_t old_conf = ctx->conf_elems[0] + ctx->conf_elems[1];
     const size_t old_queue = ctx->var_classes.size();
     bd_status s = plan(ctx);
     if (s != BD_OK) return s;
@@ -1269,9 +1300,9 @@ bd_status replan(bd_ctx* ctx)
     if ((s = dalloc(ctx, (void**)&ctx->d_part, sizeof(double) * (size_t)ctx->part_ring * (size_t)ctx->part_stride)) != BD_OK)
         return s;
     if (ctx->conf) {
-        dfree(ctx, ctx->d_conf_scratch, std::max<size_t>(2 * ctx->tsize * old_conf, 16));
+        dfree(ctx, ctx->d_conf_scratch, std::max<size_t>(ctx->tsize * old_conf, 16));
         ctx->d_conf_scratch = nullptr;
-        if ((s = dalloc(ctx, &ctx->d_conf_scratch, 2 * ctx->tsize * ctx->conf_elems)) != BD_OK) return s;
+        if ((s = dalloc(ctx, &ctx->d_conf_scratch, ctx->tsize * (ctx->conf_elems[0] + ctx->conf_elems[1]))) != BD_OK) return s;
         dfree(ctx, ctx->d_dpart, std::max<size_t>(sizeof(double) * 3 * (size_t)ctx->part_ring * (size_t)old_bpart, 16));
         ctx->d_dpart = nullptr;
         if ((s = dalloc(ctx, (void**)&ctx->d_dpart, sizeof(double) * 3 * (size_t)ctx->part_ring *
@@ -1553,7 +1584,7 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
             BD_TRY(dalloc(ctx, (void**)&ctx->d_dpart, sizeof(double) * 3 * (size_t)ctx->part_ring *
                                                           (size_t)ctx->bpart_stride));
             BD_TRY(dalloc(ctx, (void**)&ctx->d_dbead, sizeof(double) * 3 * (size_t)W * (size_t)ctx->n_beads));
-            BD_TRY(dalloc(ctx, &ctx->d_conf_scratch, 2 * ctx->tsize * ctx->conf_elems));
+            BD_TRY(dalloc(ctx, &ctx->d_conf_scratch, ctx->tsize * (ctx->conf_elems[0] + ctx->conf_elems[1])));
             BD_TRY(dalloc(ctx, (void**)&ctx->d_rgz, sizeof(double) * (size_t)W * (size_t)C));
         }
         BD_TRY(dalloc(ctx, (void**)&ctx->d_tsf, sizeof(double) * (size_t)W * (size_t)M));

@@ -61,9 +61,6 @@ constexpr int kParentThreads = 64;
 // ... of a CTA of the parent kernel for few parents: one integrating warp,
 // three that draw its noise and sample it.
 constexpr int kParentThreads2 = 128;
-// Replica bonds of a warp per spring of its tile (conf_scratch): 32 lanes of
-// one replica, or of two.
-constexpr int kConfSlots = 64;
 constexpr int kAdjThreads = 128;
 
 // One warp of the parent kernel: `count` parents, chains
@@ -121,7 +118,7 @@ struct StepParams {
     // win_per_part windows (item_range); every (item, part) is a unit of work
     int32_t n_parts, win_per_part;
     int32_t store_state, pad_store;   // this launch holds its slots' last step of the chunk
-    void* conf_scratch;         // T [warps][kConfSlots L][3] window-end bonds of a warp's replicas (Eq. 5)
+    void* conf_scratch;         // T [warps][conf_bonds][3] window-end bonds of a warp's replicas (Eq. 5)
     double dt, s_min;
     int32_t S, flags, thr_mask, bell_mask;
     uint32_t key0, key1;

@@ -39,6 +39,8 @@ inline int variant_tile(int v)
 {
     return v >= kHIBase ? 0 : v >= kLJBase ? v - kLJBase : v >= kPairBase ? v - kPairBase : v;
 }
+// Bonds of a warp's replicas at most (PersistSmem::conf_bonds): its Eq. 5 scratch.
+inline int variant_bonds(int v) { return (variant_paired(v) ? 64 : 32) * variant_tile(v); }
 
 // Hydrodynamic interaction (bd_hi.cuh; bd_hi_f32.cu, bd_hi_f64.cu): kernels,
 // their CTA size and bead limit, the dynamic shared memory of a CTA, and the

@@ -75,3 +75,45 @@ def test_conformation_needs_the_flag():
         ctx.conformation(0)
     assert e.value.status == bdra.BD_E_STATE
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", [bdra.BD_PREC_FP64, bdra.BD_PREC_FP32])
+def test_diagnostics_hold_scratch_for_the_work_not_for_the_gpu(prec):
+    """Few chains over every tile: the scratch of the window-end bonds is that of the units that run, a few hundred warps, not
+    of every warp the GPU holds for every tile."""
+    import torch
+    chains = [I.Chain(n_beads=n, n_replicas=1, spring=I.SPRING_FENE, flow=I.FLOW_SHEAR, b=40.0, rate=0.1)
+              for n in (33, 100, 150, 180, 200, 240, 270, 300, 330, 370, 400, 430, 460, 500)]
+    S, W = 5, 2
+    pos0 = I.initial_positions(I.custom(chains, 1e-3, S, S * W), seed=2)
+    held = []
+    for flags in (0, bdra.BD_FLAG_CONFORMATION):
+        ctx = bdra.Context(chains, 1e-3, S, 3, pos0, precision=prec, max_windows=W, flags=flags,
+                           stream=torch.cuda.current_stream().cuda_stream)
+        ctx.step(S * W)
+        held.append(ctx.info().device_bytes)
+        if flags:
+            got = [ctx.conformation(w) for w in range(W)]
+        ctx.close()
+    want = O.conformation(chains, 1e-3, S, S * W, 3, pos0, n_threads=4)
+    _close([np.array([g[k] for g in got]) for k in range(3)], want, 1e-10 if prec == bdra.BD_PREC_FP64 else 1e-4)
+    assert held[1] - held[0] < 16 << 20
+
+
+def test_diagnostics_of_more_units_than_the_gpu_holds():
+    """Every unit finds scratch of its own: many windows of few chains side by side, and a batch larger than the GPU, in one
+    call and a window at a time."""
+    import torch
+    for chains, W in ((_chains(), 70), ([c for c in _chains() for _ in range(150)], 3)):
+        pos0 = I.initial_positions(I.custom(chains, 1e-3, 4, 4 * W), seed=6)
+        runs = []
+        for calls in ([4 * W], [4] * W):
+            ctx = bdra.Context(chains, 1e-3, 4, 3, pos0, max_windows=W, flags=bdra.BD_FLAG_CONFORMATION,
+                               stream=torch.cuda.current_stream().cuda_stream)
+            for n in calls:
+                ctx.step(n)
+            runs.append([ctx.conformation(w) for w in range(W)])
+            ctx.close()
+        for a, b in zip(*runs):
+            for x, y in zip(a, b):
+                np.testing.assert_array_equal(x, y)
