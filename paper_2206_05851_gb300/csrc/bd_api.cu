@@ -1117,43 +1117,41 @@ bd_status upload(bd_ctx* ctx, T** dst, const std::vector<T>& v)
     return BD_OK;
 }
 
-// The float64 noise tables of a device (24 MB of constants), shared by its
-// float64 contexts: filled by the first one before it is handed out, freed
-// with the last one. The maps are never destroyed, so that a context closed
-// at process exit still finds them.
+// The float64 noise tables of a device (24 MB of constants), shared by their
+// users there (float64 contexts, calls of bd_philox_normals): filled by the
+// first one before they are handed out, freed with the last one. The maps are
+// never destroyed, so that a context closed at process exit still finds them.
 struct SharedTables { void* rad = nullptr; void* ang = nullptr; int users = 0; };
 std::mutex& tables_mutex() { static std::mutex* m = new std::mutex; return *m; }
 std::map<int, SharedTables>& tables_map() { static auto* t = new std::map<int, SharedTables>; return *t; }
 
-bd_status acquire_tables(bd_ctx* ctx)
+cudaError_t acquire_tables(int device, cudaStream_t st, const void** rad, const void** ang)
 {
     std::lock_guard<std::mutex> lock(tables_mutex());
-    SharedTables& t = tables_map()[ctx->device];
+    SharedTables& t = tables_map()[device];
     if (t.users == 0) {
         cudaError_t e = cudaMalloc(&t.rad, noise_rad_bytes());
         if (e == cudaSuccess) e = cudaMalloc(&t.ang, noise_ang_bytes());
-        if (e == cudaSuccess) e = run_noise_tables(t.rad, t.ang, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);   // other streams may read them from here on
+        if (e == cudaSuccess) e = run_noise_tables(t.rad, t.ang, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // other streams may read them from here on
         if (e != cudaSuccess) {
             cudaGetLastError();
             if (t.rad) cudaFree(t.rad);
             if (t.ang) cudaFree(t.ang);
             t = SharedTables();
-            return fail(ctx, e == cudaErrorMemoryAllocation ? BD_E_OOM : BD_E_CUDA, "noise tables: %s", cudaGetErrorString(e));
+            return e;
         }
     }
     ++t.users;
-    ctx->noise_rad = t.rad;
-    ctx->noise_ang = t.ang;
-    return BD_OK;
+    *rad = t.rad;
+    *ang = t.ang;
+    return cudaSuccess;
 }
 
-void release_tables(bd_ctx* ctx)     // after the context's stream has drained
+void release_tables(int device)     // after the user's stream has drained
 {
-    if (!ctx->noise_rad) return;
-    ctx->noise_rad = ctx->noise_ang = nullptr;
     std::lock_guard<std::mutex> lock(tables_mutex());
-    SharedTables& t = tables_map()[ctx->device];
+    SharedTables& t = tables_map()[device];
     if (--t.users > 0) return;
     cudaFree(t.rad);
     cudaFree(t.ang);
@@ -1175,7 +1173,8 @@ void release(bd_ctx* ctx)
     if (ctx->adj_stream) { cudaStreamDestroy(ctx->adj_stream); ctx->adj_stream = nullptr; }
     for (void* p : ctx->allocs) cudaFree(p);
     ctx->allocs.clear();
-    release_tables(ctx);
+    if (ctx->noise_rad) release_tables(ctx->device);
+    ctx->noise_rad = ctx->noise_ang = nullptr;
     cudaGetLastError();
 }
 
@@ -1551,7 +1550,13 @@ bd_status bd_create(const bd_config* cfg, const double* init_pos, bd_ctx** out)
     }
     for (int v = 0; v < kVariantCodes; ++v) ctx->var_cost[v] = default_variant_cost(v);
     BD_TRY(plan(ctx));
-    if (ctx->f64) BD_TRY(acquire_tables(ctx));
+    if (ctx->f64) {
+        const cudaError_t e = acquire_tables(ctx->device, ctx->stream, &ctx->noise_rad, &ctx->noise_ang);
+        if (e != cudaSuccess) {
+            s = fail(ctx, e == cudaErrorMemoryAllocation ? BD_E_OOM : BD_E_CUDA, "noise tables: %s", cudaGetErrorString(e));
+            goto failed;
+        }
+    }
     {
         const int64_t M = ctx->M, C = cfg->n_chains, W = cfg->max_windows;
         std::vector<int32_t> spring_chain(M);
@@ -2091,9 +2096,23 @@ bd_status bd_philox_normals(uint64_t seed, int64_t n, const uint32_t* ctr, int32
     uint32_t* dctr = const_cast<uint32_t*>(ctr);
     double* dout = out;
     std::vector<void*> tmp;
-    auto cleanup = [&]() { for (void* q : tmp) cudaFree(q); };
+    int device = -1;                 // its noise tables are held (float64: the integrator draws from them)
+    auto cleanup = [&]() {
+        for (void* q : tmp) cudaFree(q);
+        if (device >= 0) release_tables(device);
+    };
+    if (precision == BD_PREC_FP64) {
+        int d = 0;
+        const void *rad = nullptr, *ang = nullptr;
+        cudaError_t e = cudaGetDevice(&d);
+        if (e == cudaSuccess) e = acquire_tables(d, st, &rad, &ang);
+        if (e != cudaSuccess) { cudaGetLastError(); return e == cudaErrorMemoryAllocation ? BD_E_OOM : BD_E_CUDA; }
+        device = d;
+        p.rad_tab = (const double*)rad;
+        p.ang_tab = (const double2*)ang;
+    }
     if (!cdev) {
-        if (cudaMalloc((void**)&dctr, sizeof(uint32_t) * 4 * n) != cudaSuccess) { cudaGetLastError(); return BD_E_OOM; }
+        if (cudaMalloc((void**)&dctr, sizeof(uint32_t) * 4 * n) != cudaSuccess) { cudaGetLastError(); cleanup(); return BD_E_OOM; }
         tmp.push_back(dctr);
         if (cudaMemcpyAsync(dctr, ctr, sizeof(uint32_t) * 4 * n, cudaMemcpyHostToDevice, st) != cudaSuccess) { cleanup(); return BD_E_CUDA; }
     }

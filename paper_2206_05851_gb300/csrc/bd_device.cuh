@@ -588,6 +588,8 @@ template <bool FAST> struct Normals<float, FAST> {
     }
 };
 
+// Float64: the sign convention, and the draw by the library functions that
+// NoiseTab's tables hold (the integrator draws from those; the tests compare).
 template <bool FAST> struct Normals<double, FAST> {
     static constexpr double sign = 1.0;
     template <int H>

@@ -396,7 +396,7 @@ __global__ void normals_kernel(int64_t n, const uint32_t* ctr, StepParams p, dou
                                ctr[4 * j + 3]);
     const uint4 x = philox4x32_10_rk(c, p.rk0, p.rk1);
     T z0, z1, z2;
-    Normals<T, FAST>::draw(x, noise_half(slot), z0, z1, z2);
+    draw_half<T, FAST, -1>(x, noise_half(slot), p, z0, z1, z2);
     const T sg = Normals<T, FAST>::sign;      // undo the fast path's sign flip
     out[3 * j] = (double)(sg * z0); out[3 * j + 1] = (double)(sg * z1); out[3 * j + 2] = (double)(sg * z2);
 }

@@ -1,4 +1,5 @@
-"""The integrator's float64 device functions against what they stand for: the FENE floor taken by the bits of s against the
+"""The integrator's float64 device functions against what they stand for: the tabulated normals against Box-Muller by the
+library functions (every 21-bit field, bit for bit), the FENE floor taken by the bits of s against the
 comparison it replaces, the reciprocal of the pair forces against the division."""
 import ctypes
 import os
@@ -33,6 +34,40 @@ def dev():
 
 def _p(a):
     return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def test_tabulated_normals_are_the_library_functions_bits(dev):
+    bad = ctypes.c_ulonglong(1)
+    assert dev.check_noise(ctypes.byref(bad)) == 0
+    assert bad.value == 0
+
+
+def test_noise_diagnostic_shares_the_tables_and_gives_them_back():
+    """bd_philox_normals draws as the integrator does, from the tables: the same values with and without a float64 context
+    that holds them, which reads them after a call, and no memory kept when the last user is gone."""
+    import torch
+    ctr = np.random.default_rng(1).integers(0, 2 ** 24, size=(5000, 4)).astype(np.uint32)
+    out = [np.zeros((5000, 3)) for _ in range(3)]
+    torch.cuda.synchronize()
+    bdra.bd_philox_normals(5, ctr, bdra.BD_PREC_FP64, out[0])
+    free = torch.cuda.mem_get_info()[0]
+    bdra.bd_philox_normals(5, ctr, bdra.BD_PREC_FP64, out[1])
+    assert torch.cuda.mem_get_info()[0] == free
+    chains = [I.Chain(n_beads=12, n_replicas=3, spring=I.SPRING_FENE, flow=I.FLOW_SHEAR, b=30.0, rate=0.1)]
+    wl = I.custom(chains, 1e-3, 5, 10)
+    runs = []
+    for ask in (False, True):
+        ctx = bdra.Context(chains, wl.dt, 5, 1, I.initial_positions(wl, seed=3), precision=bdra.BD_PREC_FP64, max_windows=2,
+                           stream=torch.cuda.current_stream().cuda_stream)
+        ctx.step(5)
+        if ask:
+            bdra.bd_philox_normals(5, ctr, bdra.BD_PREC_FP64, out[2])
+        ctx.step(5)
+        runs.append(ctx.positions(True))
+        ctx.close()
+    np.testing.assert_array_equal(runs[0], runs[1])
+    np.testing.assert_array_equal(out[0], out[1])
+    np.testing.assert_array_equal(out[0], out[2])
 
 
 @pytest.mark.parametrize("Hinvb", [1.0, 0.25, 0.0])
