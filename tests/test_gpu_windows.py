@@ -146,3 +146,27 @@ def test_event_list_and_survival_at_the_edges_of_the_one_cta_form(beads):
         np.testing.assert_allclose(surv[c], s, rtol=ch.n_beads * 2.0 ** -52)     # another order of the sum
         at += ch.n_beads - 1
     np.testing.assert_array_equal(dev_surv.cpu().numpy(), surv)
+
+
+@pytest.mark.parametrize("prec", [bdra.BD_PREC_FP32, bdra.BD_PREC_FP64])
+@pytest.mark.parametrize("batch", sorted(BATCHES))
+def test_overlapped_schedule_equals_parents_first(batch, prec):
+    """Parents beside replicas (small batches, chains with hydrodynamic interaction) and parents before replicas (while the two
+    are timed) give the same bits on equal calls: over several windows, one window, a start and an end inside a window."""
+    chains = BATCHES[batch]
+    if batch == "many" and prec == bdra.BD_PREC_FP64:
+        chains = chains[:24]
+    S, W = 6, 8
+    wl = I.custom(chains, 4e-5 if chains[0].spring == I.SPRING_HARMONIC else 1e-3, S, S * W)
+    got = []
+    for timing in (False, True):
+        ctx = bdra.Context(chains, wl.dt, S, 11, I.initial_positions(wl, seed=5), precision=prec, max_windows=W,
+                           thr_mask=7, bell_mask=7, stream=torch.cuda.current_stream().cuda_stream)
+        bdra.bd_enable_timing(ctx.ptr, timing)
+        for n in (3 * S, S, 2, S + 3, S + 1):
+            ctx.step(n)
+        got.append([ctx.replica_average(w) for w in range(7)] + [ctx.time_average(w) for w in range(7)] +
+                   [ctx.positions(True), *ctx.kinetics(), np.array(ctx.info().overextensions)])
+        ctx.close()
+    for a, b in zip(*got, strict=True):
+        np.testing.assert_array_equal(a, b)
