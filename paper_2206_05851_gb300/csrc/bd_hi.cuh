@@ -246,8 +246,7 @@ __device__ __forceinline__ void hi_load_tiles(HITiles<T, MAXT>& tl, const HIShar
 }
 
 // Factor of a diagonal tile (lower part; the upper part is left as is) and
-// the reciprocals of its diagonal. The fast float form takes both from one
-// approximate reciprocal square root.
+// the reciprocals of its diagonal, both from one reciprocal square root.
 template <typename T, bool FAST>
 __device__ __forceinline__ void hi_chol4(T (&A)[16], T (&inv)[4])
 {
@@ -256,15 +255,8 @@ __device__ __forceinline__ void hi_chol4(T (&A)[16], T (&inv)[4])
         T s = A[5 * j];
 #pragma unroll
         for (int k = 0; k < j; ++k) s = fma(-A[4 * j + k], A[4 * j + k], s);
-        T l, il;
-        if (FAST) {
-            il = Rsqrt<T, FAST>::rsqrt(s);
-            l = s * il;
-        } else {
-            l = sqrt(s);
-            il = T(1) / l;
-        }
-        A[5 * j] = l;
+        const T il = Rsqrt<T, FAST>::rsqrt(s);
+        A[5 * j] = s * il;
         inv[j] = il;
 #pragma unroll
         for (int i = j + 1; i < 4; ++i) {
@@ -653,26 +645,6 @@ template <int NTM> struct HIShared64 {
     double com[3];
 };
 
-__device__ __forceinline__ void hi_chol4_64(double (&A)[16], double (&inv)[4])
-{
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        double s = A[5 * j];
-#pragma unroll
-        for (int k = 0; k < j; ++k) s = fma(-A[4 * j + k], A[4 * j + k], s);
-        const double il = rsqrt(s);
-        A[5 * j] = s * il;
-        inv[j] = il;
-#pragma unroll
-        for (int i = j + 1; i < 4; ++i) {
-            double v = A[4 * i + j];
-#pragma unroll
-            for (int k = 0; k < j; ++k) v = fma(-A[4 * i + k], A[4 * j + k], v);
-            A[4 * i + j] = v * il;
-        }
-    }
-}
-
 // hi_cholesky on the shared tiles.
 template <int NTM>
 __device__ __forceinline__ void hi_cholesky64(HIShared64<NTM>& sm, int NT)
@@ -680,7 +652,7 @@ __device__ __forceinline__ void hi_cholesky64(HIShared64<NTM>& sm, int NT)
     const int tid = threadIdx.x, total = NT * (NT + 1) / 2;
     auto diagonal = [&](double (&A)[16], int t) {
         double inv[4];
-        hi_chol4_64(A, inv);
+        hi_chol4<double, false>(A, inv);
         hi_st16(sm.diag, A);
 #pragma unroll
         for (int e = 0; e < 4; ++e) sm.dinv[e] = inv[e];

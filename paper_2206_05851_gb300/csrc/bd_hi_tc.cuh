@@ -543,7 +543,6 @@ __device__ __forceinline__ void hi_tc_begin(HITCShared& sm, TCState& ts, int N)
         tc::mbar_init(&sm.bar_next, 1);
         tc::mbar_init(&sm.bar_rest, 1);
     }
-    for (int e = threadIdx.x; e < 128 * 32; e += blockDim.x) sm.op_hi[e] = sm.op_lo[e] = 0.0f;
     tc_pairs_init(sm, N, N > 42 ? N - 42 : 0);
     if (warp == 0) {
         tc::tmem_alloc(&sm.taddr, kTCCols);
