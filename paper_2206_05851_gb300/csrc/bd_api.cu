@@ -378,7 +378,7 @@ int64_t parent_warps_at(const bd_ctx* ctx, int least)
     return warps;
 }
 // Up to how many warps of parents an SM the block kernel is the faster one
-// (us a step): 64 float64 chains of 100 beads 27.5 -> 4.8, 256 float32 chains
+// (us a step): 64 float64 chains of 100 beads 27.5 -> 4.3, 256 float32 chains
 // of 100 beads 1.11 -> 0.65, 512 of 20 to 500 beads 7.1 -> 2.8; 1024 of 100
 // beads 1.34 -> 1.45, 16384 of 50 beads with every criterion 7.2 -> 14.8.
 constexpr int kParentBlockWarps = 5;

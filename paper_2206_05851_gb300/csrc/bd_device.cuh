@@ -83,7 +83,7 @@ enum { BD_DEV_ERR_TC_WAIT = 1 };   // a tensor-core completion wait gave up
 
 struct StepParams {
     const ChainDev* chains;
-    const ItemDev* items;       // replica kernel: warp work items, longest first
+    const ItemDev* items;       // replica kernel: warp work items of its variant, first noise half first (order_items)
     int32_t n_items;
     int32_t* queue;             // [n_parts] work items claimed (zeroed before each launch)
     const int32_t* parent_items;  // parent kernel: chain ids

@@ -7,13 +7,14 @@
 // neighbouring lanes are reached with warp shuffles, so a step touches neither
 // shared nor global memory.
 //
-// Two kernels share one step routine:
+// Two kernels share one step routine (step_bonds; collapsed chains: step_bonds_lj):
 //   parent_kernel  advances every parent, writes its conformation at each
 //                  window end (the "halted parent" that the next window's
 //                  replicas copy; bd_set_positions writes the first), and
 //                  samples it every step (ISF criteria, TSF sums); few
 //                  parents run on parent_block_kernel instead;
-//   replica_kernel one CTA per (chain, replica group) evolves the replicas
+//   replica_persist_kernel (bd_persist.cuh): warps claim (chain, replica
+//                  group) items over runs of windows and evolve their replicas
 //                  window after window: spawn from the parent snapshot, S
 //                  steps, one force sample per replica at the window end,
 //                  float64 cross-replica sum.
