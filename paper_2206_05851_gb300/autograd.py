@@ -10,7 +10,7 @@ is argument marshalling; the forward and backward work runs in the library's
 kernels, on torch's current CUDA stream.
 
 Device memory. The run's context (state, histories, parent checkpoints and,
-after the first backward, the adjoint's replay buffers: about 3.4 GB for 256
+after the first backward, the adjoint's replay buffers: about 4 GB for 256
 chains of 200 beads) is held by the autograd graph only until its backward
 pass, which releases it, the way autograd frees saved tensors. A second
 backward through the same graph then raises; set ``RunSpec.retain_run`` to
